@@ -15,6 +15,7 @@
 // unknown (stage value) or a strip node holding a bulk node's macros at t
 // and t + 1 (interpolated linearly at the stage time, Sec. 3.3).
 #include "charsys.cuh"
+#include "ff.cuh"
 
 #include <algorithm>
 #include <cooperative_groups.h>
@@ -167,66 +168,6 @@ __device__ __forceinline__ void put_async(unsigned a, double v, unsigned bar)
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
                  ::"r"(a), "l"(__double_as_longlong(v)), "r"(bar) : "memory");
-}
-
-// Unevaluated sums hi + lo of two floats ("float-float"), built from the
-// error-free transformations TwoSum (Knuth) and TwoProduct (by FMA): about
-// 48 significant bits at FP32 issue cost.  The band kernel forms the wave
-// amplitudes and the right-hand side with FP32 and FP16 storage in them
-// instead of FP64 (one FP64 warp instruction per 64 cycles on each SM
-// sub-partition; with the four components of a tile on one SM the FP64
-// work would queue there): their projections S dU/dn cancel (an acoustic
-// wave has a small entropy part), and plain FP32 lost accuracy there.
-struct FF {
-    float h, l;
-};
-__device__ __forceinline__ FF ff_fast(float a, float b)      // |a| >= |b|
-{
-    const float s = a + b;
-    return {s, b - (s - a)};
-}
-__device__ __forceinline__ FF ff_two_sum(float a, float b)
-{
-    const float s = a + b, z = s - a;
-    return {s, (a - (s - z)) + (b - z)};
-}
-__device__ __forceinline__ FF ff_prod(float a, float b)
-{
-    const float p = a * b;
-    return {p, fmaf(a, b, -p)};
-}
-__device__ __forceinline__ FF ff_add(FF x, FF y)
-{
-    const FF s = ff_two_sum(x.h, y.h), t = ff_two_sum(x.l, y.l);
-    const FF u = ff_fast(s.h, s.l + t.h);
-    return ff_fast(u.h, u.l + t.l);
-}
-__device__ __forceinline__ FF ff_neg(FF x) { return {-x.h, -x.l}; }
-__device__ __forceinline__ FF ff_mul(FF x, float b)
-{
-    const FF p = ff_prod(x.h, b);
-    return ff_fast(p.h, fmaf(x.l, b, p.l));
-}
-__device__ __forceinline__ FF ff_mul(FF x, FF y)
-{
-    const FF p = ff_prod(x.h, y.h);
-    return ff_fast(p.h, fmaf(x.h, y.l, fmaf(x.l, y.h, p.l)));
-}
-__device__ __forceinline__ double ff_to_double(FF x) { return double(x.h) + double(x.l); }
-__device__ __forceinline__ double ff_pack(FF x)
-{
-    return __hiloint2double(__float_as_int(x.h), __float_as_int(x.l));
-}
-__device__ __forceinline__ FF ff_unpack(double v)
-{
-    return {__int_as_float(__double2hiint(v)), __int_as_float(__double2loint(v))};
-}
-__device__ __forceinline__ FF ff_const(const float (&c)[2]) { return {c[0], c[1]}; }
-__device__ __forceinline__ FF ff_scale(FF x, float p2) { return {x.h * p2, x.l * p2}; }   // p2: a power of 2
-__device__ __forceinline__ FF ff_split(double d)
-{
-    const float h = float(d);
-    return {h, float(d - double(h))};
 }
 
 // v into slot p of every CTA of the cluster, counted on barrier `bar` there
