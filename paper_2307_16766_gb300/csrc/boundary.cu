@@ -27,26 +27,19 @@ namespace lbmgb {
 namespace {
 
 constexpr int kBandThreads = 32;   // allocation-free path: one thread per unknown
-// Fused band kernel: a group of kTileThreads threads per characteristic
-// component, one thread per local unknown of the tile.
+// Fused band kernel: a thread per local unknown of the tile (and, with FP64
+// storage, per characteristic component: kCluster CTAs).
 constexpr int kTileThreads = kTileUnknowns;
-constexpr int kCluster = 4;         // groups per band tile: one per characteristic component
-
-// A band tile is, with FP32 / FP16 storage (MONO), one CTA of kCluster
-// groups (the whole tile on one SM), and with FP64 storage a cluster of
-// kCluster CTAs of one group each (one SM per characteristic component).
-template <bool MONO>
-constexpr int band_threads() { return MONO ? kCluster * kTileThreads : kTileThreads; }
+constexpr int kCluster = 4;
 
 // ---------------------------------------------------------------------------
-// The band kernel: four component groups per tile
+// The band kernel
 // ---------------------------------------------------------------------------
-// Group r owns component / wave r of every unknown of the tile.  With FP64
-// storage (one warp instruction of FP64 per 64 cycles on each SM
-// sub-partition) the groups are the four CTAs of a cluster on four SMs,
-// exchanging their shares through distributed shared memory; with FP32 /
-// FP16 storage the wave arithmetic is float-float and the four groups share
-// one CTA and its shared memory.
+// FP32 / FP16 storage: one CTA per tile, a thread per unknown
+// (band_tile_mono).  FP64 storage: one warp instruction of FP64 takes 64
+// cycles on each SM sub-partition, so a tile is a cluster of four CTAs on
+// four SMs, CTA r forming component / wave r of every unknown and exchanging
+// through distributed shared memory (band_tile).
 
 // Share c of the mesoscopic viscous vector (see vis_meso), in arithmetic
 // type R: V1 for c = 1, V2 for c = 2; V3 is split, its conductive part for
@@ -214,11 +207,334 @@ __device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
 __device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
 
-// One tile of the boundary band: a run of positions of one characteristic
-// side (all M layers, and the corner next to it on a W/E side), plus the
-// halo its four RK4 stages need (Sec. 3.3).  Four groups of 128 threads
-// (MONO: one CTA; FP64: a cluster of four CTAs), group r forming wave r and
-// lab component r of every local unknown.
+// S row products, RK4 sums and frames in float-float, for the one-CTA tile.
+__device__ __forceinline__ FF ff_addf(FF x, float b)
+{
+    const FF s = ff_two_sum(x.h, b);
+    return ff_fast(s.h, s.l + x.l);
+}
+
+// One tile of the boundary band with FP32 / FP16 storage, in one CTA: the
+// phases of band_tile below (strip nodes, the four RK4 stages of the tile's
+// unknowns in shared memory, the Dirichlet write), with one thread carrying
+// an unknown's whole right-hand side, all four waves and components in
+// registers (float-float, see ff.cuh).
+//
+// What bounds it is latency: the strip's global round trips, then four
+// dependent stages of ~900 FP32 instructions on one warp per SM
+// sub-partition, one barrier each (the stage values a neighbour reads are
+// double-buffered).  With an unknown's four components on four threads (the
+// form before this one) the inputs of the system were formed four times and
+// every stage had two barriers and an exchange: a step of the 256^2 pulse
+// (32 tiles) took 24.0 us, now 20.7 us.
+//
+// WIDE (a grid's own band launch): 512 threads, the whole SM, which keeps
+// the bulk kernel's CTAs off it.  Warps 0-3 carry the unknowns; warps 0-7
+// pull the strip nodes; meanwhile warps 8-15 run one stage and the Dirichlet
+// write without effect, each one part of that code, so that it is in the
+// SM's instruction caches when warps 0-3 get there (the stage code otherwise
+// arrives line by line under the bulk kernel's traffic).  Otherwise (many
+// tiles in one launch): 128 threads, four CTAs resident per SM, one tile's
+// round trips beside the others' stages; the code stays cached from tile to
+// tile.
+template <int LAT, typename S, bool REF, bool WIDE>
+__device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, const Band& B, const Export& E,
+                                               const S* __restrict__ fin, S* __restrict__ f, int par_t, int tile)
+{
+    using L = Lat<LAT>;
+    using C = typename Store<S>::C;
+    constexpr bool TH = L::THERMAL;
+    // a kernel launched after this one for early start (the bulk update,
+    // which reads only the old buffer) may begin now
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int kPull = WIDE ? 2 * kTileThreads : kTileThreads;      // threads of the strip phase
+    const int tid = int(threadIdx.x), l = tid % kTileThreads, warp = tid / 32;
+    const bool dry = WIDE && warp >= kPull / 32;
+    __shared__ __align__(16) float Ys[2][kTileThreads * 4];     // stage values, lab frame
+    extern __shared__ __align__(16) unsigned char dyn_raw[];
+    float* SUt = reinterpret_cast<float*>(dyn_raw);    // [max_nodes][4] macros of t
+    float* SUt1 = SUt + 4 * B.max_nodes;               // [max_nodes][4] macros of t + 1
+    float* SNt = SUt1 + 4 * B.max_nodes;               // [max_nodes][5] moments of t
+    S* Fx = reinterpret_cast<S*>(SNt + 5 * B.max_nodes);   // [max_fx][Q]
+    const int ns = B.max_nodes;
+    const UDesc D = B.ld[(long long)tile * kTileUnknowns + l];
+    const int lev = D.level;            // > 4: no unknown on this thread
+    const bool meso = B.viscous == VIS_MESO;
+    const bool carrier = !WIDE || warp < kTileThreads / 32;
+    double U0d[4] = {0.0, 0.0, 0.0, 0.0};
+
+    // 1. strip nodes: macros of t and moments of t loaded, macros of t + 1
+    // pulled (Eqs. lbe, macro); post-collision populations of Eq. NEEP sources
+    // kept.  The nodes are dealt round the warps.
+    if (!dry) {
+        const StripNode* snt = B.sn + (long long)tile * ns;
+        const float* gU = static_cast<const float*>(E.stripU) + (long long)par_t * E.nslots * 4;
+        const float* gN = static_cast<const float*>(E.stripN) + (long long)par_t * E.nslots * 5;
+        const int k0 = (kPull / 32) * (tid % 32) + warp;
+        StripNode N0{-1, -1, 0, -1, -1, 0};
+        if (k0 < ns) N0 = snt[k0];
+        if (carrier && lev <= 4) {
+            const double2* p = reinterpret_cast<const double2*>(B.Ub + ((long long)par_t * B.n_unk + D.gid) * 4);
+            const double2 a = p[0], b = p[1];
+            U0d[0] = a.x; U0d[1] = a.y; U0d[2] = b.x; U0d[3] = b.y;
+        }
+#pragma unroll 1
+        for (int k = k0; k < ns; k += kPull) {
+            const StripNode N = N0;
+            const int kn = k + kPull;
+            if (kn < ns) N0 = snt[kn];      // the next node's descriptor beside this one's pull
+            if (N.x < 0) continue;
+            if (N.flags & kSNLoadT) {
+                const float4 u = *reinterpret_cast<const float4*>(gU + 4LL * N.tslot);
+                *reinterpret_cast<float4*>(SUt + 4 * k) = u;
+                if (meso) {
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) SNt[5 * k + c] = gN[5LL * N.tslot + c];
+                }
+            }
+            if (!(N.flags & kSNPull)) continue;
+            C g[L::Q];
+            pull_plain<LAT, S, C>(G, O, fin, N.x, N.y, g);
+            if (Store<S>::SCALED) {
+#pragma unroll
+                for (int i = 0; i < L::Q; ++i) g[i] *= C(L::w(i));
+            }
+            Moments<LAT, C> m;
+            if (N.fx >= 0) {
+                S* fx = Fx + N.fx * L::Q;
+                m = collide<LAT, C, REF>(G, g, [&](int i, C v) {
+                    if (Store<S>::SCALED) v *= C(1.0 / L::w(i));
+                    Store<S>::put(fx + i, v);
+                });
+            } else {
+                m = moments_G<LAT, C, REF>(G, g);
+            }
+            const float4 u1 = make_float4(m.s0, m.ux, m.uy, m.dT);
+            *reinterpret_cast<float4*>(SUt1 + 4 * k) = u1;
+            if (N.gslot >= 0) {             // the strips of t + 1, for the next step
+                const long long slot = (long long)(par_t ^ 1) * E.nslots + N.gslot;
+                *reinterpret_cast<float4*>(static_cast<float*>(E.stripU) + slot * 4) = u1;
+                if (N.flags & kSNNeq) {     // a node of the mesoscopic stencil
+                    float N1[5];
+                    neq_moments<LAT, C, float>(g, m, 1.0f - 0.5f * omega_of<float>(G), N1);
+                    float* q = static_cast<float*>(E.stripN) + slot * 5;
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) q[c] = N1[c];
+                }
+            }
+        }
+        if (carrier && lev <= 4)
+            *reinterpret_cast<float4*>(Ys[0] + 4 * l) =
+                make_float4(float(U0d[0]), float(U0d[1]), float(U0d[2]), float(U0d[3]));
+    }
+    if (!dry) {
+        if (WIDE) asm volatile("bar.sync 1, %0;" ::"n"(2 * kTileThreads) : "memory");
+        else __syncthreads();
+        if (!carrier) return;               // a helper of the strip phase
+    }
+
+    // 2. RK4 (Sec. 3.3).  part: what a warm-up warp runs (0: stencils and
+    // inputs, 1: the viscous vector, 2: the waves, 3: the right-hand side and
+    // RK4 update, 4: the Dirichlet write, 5: none); 8: all of it
+    const int part = dry ? warp - kPull / 32 : 8;
+    CtxT<float> X;
+    X.St = SUt;
+    X.St1 = SUt1;
+    const float rho0r = rho0_of<float>(G), cs2r = float(L::CS2), kr = B.kR_f;
+    const bool side = lev <= 4 && D.kind < 4, corner = lev <= 4 && !side;
+    const int scheme = side ? B.scheme[D.kind] : SCH_LODI;
+    const bool cbc = scheme == SCH_CBC || scheme == SCH_CBC_RELAX;
+    const bool vis = B.viscous != VIS_OFF;
+    // the incoming wave of a scheme is fT S T + c + fV S V (+ beta (P - P_inf)
+    // on acoustic waves): Eq. LODI-Relax (-alpha_T, alpha_T t_inf, 0), Eq.
+    // CBC-PNR (1, 0, 1), Eq. CBC-Relax (1 - alpha_T, alpha_T t_inf, 1 - alpha_V)
+    const FF one{1.0f, 0.0f}, zero{0.0f, 0.0f};
+    const bool relax = scheme == SCH_LODI_RELAX || scheme == SCH_CBC_RELAX;
+    const FF fT = scheme == SCH_CBC_RELAX ? ff_const(B.ffk[FFK_1MAT])
+                : scheme == SCH_LODI_RELAX ? ff_neg(ff_const(B.ffk[FFK_AT])) : one;
+    const FF fV = scheme == SCH_CBC_RELAX ? ff_const(B.ffk[FFK_1MAV]) : one;
+    const FF cI = relax ? ff_const(B.ffk[FFK_ATTI]) : zero;
+    FF u0[4], acc[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        u0[m] = ff_split(U0d[m]);
+        acc[m] = zero;
+    }
+    int mask = 0;                       // incoming waves of time t
+    float V[4] = {0, 0, 0, 0};          // viscous vector (local frame, frozen)
+    float Ynew[4] = {0, 0, 0, 0};
+#pragma unroll 1
+    for (int stage = 0; stage < (dry ? 1 : 4); ++stage) {
+        X.Y = Ys[stage & 1];
+        X.frac = stage == 0 ? 0.0f : (stage == 3 ? 1.0f : 0.5f);
+        if (lev <= 3 - stage) {
+            const int kind = D.kind;
+            float Ul[4] = {0, 0, 0, 0}, dUn[4] = {0, 0, 0, 0}, TT[4] = {0, 0, 0, 0};
+            float irho = 0, sth = 0, isth = 0, dP = 0;
+            // inputs of the system: dU/dn, 1/rho, sqrt(theta), 1/sqrt(theta),
+            // P - P_inf and the transversal terms
+            if (part == 8 || part == 0) {
+                float A[4], Bv[4];
+                fetch_local(X, l, kind, kr, Ul);
+                irho = 1.0f / (rho0r + Ul[0]);
+                if (TH) {
+                    sth = sqrtf(1.0f + Ul[3]);
+                    isth = rsqrtf(1.0f + Ul[3]);
+                }
+                // normal derivative: one-sided at the outermost layer (Eq.
+                // FD-dx-bw) and along a corner's diagonal (spacing sqrt 2),
+                // central at inner layers (Eq. FD-dx-center)
+                const bool one_sided = corner || D.j == B.M;
+                fetch_local(X, side && one_sided ? D.nb[1] : D.nb[0], kind, kr, A);
+                fetch_local(X, side && one_sided ? D.nb[2] : D.nb[1], kind, kr, Bv);
+                const float kn = corner ? B.kC_f : 0.5f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+                    dUn[m] = (one_sided ? 3.0f * Ul[m] - 4.0f * A[m] + Bv[m] : A[m] - Bv[m]) * kn;
+                if (side) {
+                    float Up[4], Um[4];
+                    fetch_local(X, D.nb[4], kind, kr, Up);
+                    fetch_local(X, D.nb[5], kind, kr, Um);
+                    TT[0] = -0.5f * ((rho0r + Up[0]) * Up[2] - (rho0r + Um[0]) * Um[2]);
+                    TT[1] = -Ul[2] * (0.5f * (Up[1] - Um[1]));
+                    // rho T - rho0 = drho + rho0 dT + drho dT
+                    const float d6 = TH ? 0.5f * ((Up[0] + rho0r * Up[3] + Up[0] * Up[3]) -
+                                                  (Um[0] + rho0r * Um[3] + Um[0] * Um[3]))
+                                        : 0.5f * (Up[0] - Um[0]);
+                    TT[2] = -cs2r * irho * d6 - Ul[2] * (0.5f * (Up[2] - Um[2]));
+                    if (TH) TT[3] = -0.5f * ((1.0f + Up[3]) * Up[2] - (1.0f + Um[3]) * Um[2]);
+                    dP = (TH ? cs2r * (Ul[0] + rho0r * Ul[3] + Ul[0] * Ul[3]) : cs2r * Ul[0]) - B.pdev_f[kind];
+                }
+            }
+            if (stage == 0 && side && (part == 8 || part == 1)) {
+                float Vc[4] = {0, 0, 0, 0};
+                if (B.viscous == VIS_FD) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) Vc[c] = vis_fd_c<TH, float>(c, G, B, X, D, l, cs2r);
+                } else if (B.viscous == VIS_MESO) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) Vc[c] = vis_meso_c<TH, float>(c, G, SUt, SNt, D, cs2r);
+                }
+                V[1] = Vc[1];
+                V[2] = Vc[2];
+                V[3] = TH ? Vc[0] + Vc[3] : 0.0f;       // V0 = 0; V3 from two shares
+            }
+            // the waves: row i of S applied to dU/dn (outgoing, times
+            // Lambda_i) or to T and V (incoming).  Rows: thermal (-r/2, 0, 0, 1/2),
+            // (0, 0, 1, 0), (r/4, -+a, 0, 1/4); isothermal (1/2, -+h, 0), (0, 0, 1)
+            FF w[4] = {zero, zero, zero, zero};
+            if (part == 8 || part == 2) {
+                const float rr = TH ? (1.0f + Ul[3]) * irho : 0.0f;
+                const float c1 = TH ? sth * B.kA_f : (rho0r + Ul[0]) * B.ihcs_f;
+                const float cw = TH ? sth * B.kB_f : B.cs_f;
+                auto row = [&](int i, const float* v) -> FF {
+                    if (i == 1) return FF{v[2], 0.0f};
+                    if (TH) {
+                        if (i == 0) return ff_add(ff_prod(-0.5f * rr, v[0]), ff_prod(0.5f, v[3]));
+                        return ff_add(ff_add(ff_prod(0.25f * rr, v[0]), ff_prod(0.25f, v[3])),
+                                      ff_prod(i == 2 ? -c1 : c1, v[1]));
+                    }
+                    return ff_add(ff_prod(0.5f, v[0]), ff_prod(i == 0 ? -c1 : c1, v[1]));
+                };
+#pragma unroll
+                for (int i = 0; i < (TH ? 4 : 3); ++i) {
+                    const bool acoustic = TH ? i >= 2 : i != 1;
+                    const float lam = !acoustic ? Ul[1] : Ul[1] + ((i == 2) == TH ? -cw : cw);
+                    if (stage == 0 && (dry ? (l & 1) != 0 : lam < 0.0f)) mask |= 1 << i;
+                    const bool inc = (mask >> i) & 1;
+                    float v[4];
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) v[m] = inc ? TT[m] : dUn[m];
+                    const FF s = row(i, v);
+                    if (!inc) {
+                        w[i] = ff_mul(s, lam);
+                    } else if (scheme != SCH_LODI) {
+                        FF x = scheme == SCH_CBC ? s : ff_add(ff_mul(s, fT), cI);
+                        if (cbc && vis) {
+                            const FF sv = row(i, V);
+                            x = ff_add(x, scheme == SCH_CBC ? sv : ff_mul(sv, fV));
+                        }
+                        if (acoustic && relax) x = ff_add(x, ff_mul(ff_const(B.ffk[FFK_BP]), dP));
+                        w[i] = x;
+                    }
+                }
+            }
+            if (part == 8 || part == 3) {
+                // -S^-1 w (+ T + V for the CBC schemes), with r^-1 = rho /
+                // theta and b = sqrt(2 c_s^4 / T~)
+                FF k[4];
+                if (TH) {
+                    const FF w23 = ff_add(w[2], w[3]);
+                    k[0] = ff_neg(ff_mul(ff_sub(w23, w[0]), (rho0r + Ul[0]) * isth * isth));
+                    k[1] = ff_neg(ff_mul(ff_sub(w[3], w[2]), isth * B.kB_f));
+                    k[3] = ff_neg(ff_add(w23, w[0]));
+                } else {
+                    k[0] = ff_neg(ff_add(w[0], w[2]));
+                    k[1] = ff_neg(ff_mul(ff_sub(w[2], w[0]), B.cs_f * irho));
+                    k[3] = zero;
+                }
+                k[2] = ff_neg(w[1]);
+                if (cbc) {
+                    k[0] = ff_addf(k[0], TT[0]);
+                    k[1] = ff_addf(k[1], TT[1] + V[1]);
+                    k[2] = ff_addf(k[2], TT[2] + V[2]);
+                    if (TH) k[3] = ff_addf(k[3], TT[3] + V[3]);
+                }
+                // to the lab frame
+                if (side) {
+                    const FF n = (kind == 0 || kind == 2) ? ff_neg(k[1]) : k[1], t = k[2];
+                    k[1] = kind < 2 ? n : t;
+                    k[2] = kind < 2 ? t : n;
+                } else {
+                    const int c = kind - 4;
+                    const FF r = ff_const(B.ffk[FFK_KR]);
+                    const FF n0 = (c & 1) ? r : ff_neg(r), n1 = (c & 2) ? r : ff_neg(r), n = k[1], t = k[2];
+                    k[1] = ff_sub(ff_mul(n, n0), ff_mul(t, n1));
+                    k[2] = ff_add(ff_mul(n, n1), ff_mul(t, n0));
+                }
+                // RK4: U(t + 1) = U(t) + (k1 + 2 k2 + 2 k3 + k4) / 6
+                const float hk = stage == 2 ? 1.0f : 0.5f, wk = stage == 0 ? 1.0f : 2.0f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    FF y;
+                    if (stage < 3) {
+                        acc[m] = ff_add(acc[m], ff_scale(k[m], wk));
+                        y = ff_add(u0[m], ff_scale(k[m], hk));
+                    } else {
+                        y = ff_add(u0[m], ff_mul(ff_add(acc[m], k[m]), ff_const(B.ffk[FFK_SIXTH])));
+                        U0d[m] = ff_to_double(y);
+                    }
+                    Ynew[m] = y.h;
+                }
+                if (!dry && stage < 3)
+                    *reinterpret_cast<float4*>(Ys[(stage & 1) ^ 1] + 4 * l) =
+                        make_float4(Ynew[0], Ynew[1], Ynew[2], Ynew[3]);
+            }
+        }
+        if (!dry && stage < 3) {
+            if (WIDE) asm volatile("bar.sync 2, %0;" ::"n"(kTileThreads) : "memory");
+            else __syncthreads();
+        }
+    }
+
+    // 3. U(t + 1) and the Dirichlet populations of the owned unknowns
+    if (lev == 0 && (part == 8 || part == 4)) {
+        if (!dry) {
+            double2* p = reinterpret_cast<double2*>(B.Ub + ((long long)(par_t ^ 1) * B.n_unk + D.gid) * 4);
+            p[0] = make_double2(U0d[0], U0d[1]);
+            p[1] = make_double2(U0d[2], U0d[3]);
+        }
+        const bool neep = B.dirichlet >= 1;     // needs x_f: NEEP or regularised NEEP
+        dirichlet<LAT, S, float, REF>(G, B, f, neep ? SUt1 + 4 * D.wslot : nullptr,
+                                      neep ? Fx + D.wsrc * L::Q : nullptr, D, Ynew, dry);
+    }
+}
+
+// One tile of the boundary band with FP64 storage: a run of positions of one
+// characteristic side (all M layers, and the corner next to it on a W/E
+// side), plus the halo its four RK4 stages need (Sec. 3.3).  A cluster of
+// four CTAs of 128 threads, CTA r forming wave r and lab component r of every
+// local unknown.
 //
 // 1. Strip nodes: the tile pulls the bulk nodes at depths 0..2 next to the
 //    side that its stencils read (Eq. lbe) for their macros at t + 1
@@ -237,7 +553,7 @@ __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
 //    mask of time t.
 // 3. The owners write U(t + 1) and the mesoscopic Dirichlet populations
 //    (equilibrium or Eq. NEEP), shared out over the four groups.
-template <int LAT, typename S, bool REF, bool MONO>
+template <int LAT, typename S, bool REF>
 __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const Band& B,
                                           const Export& E, const S* __restrict__ fin,
                                           S* __restrict__ f, int par_t, int tile)
@@ -249,22 +565,9 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     // a kernel launched after this one for early start (the bulk update,
     // which reads only the old buffer) may begin now
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // MONO (FP32 / FP16 storage): one CTA of four 128-thread groups per
-    // tile, group r in the role of cluster rank r, exchanging through its
-    // own shared memory (the tile then holds one SM and leaves the others to
-    // the bulk kernel); FP64 storage: a cluster of four 128-thread CTAs.
-    static_assert(!MONO || sizeof(S) < 8, "FP64 storage keeps the cluster form");
-    const int grp = MONO ? int(threadIdx.x / kTileThreads) : int(cg::this_cluster().block_rank());
-    const int l = int(threadIdx.x % kTileThreads);
-    // MONO: groups 0 and 1 do the strip phase for the tile; meanwhile the
-    // eight warps of groups 2 and 3 run one stage and the Dirichlet write
-    // without effect (no stores, no waits), each warp one part of that code
-    // with its lanes in all four roles, so that the code is in the SM's
-    // instruction caches when the tile reaches it (measured: the first
-    // stage otherwise waits several microseconds on instruction fetch under
-    // the bulk kernel's traffic, and one warp fetching it all in sequence
-    // takes longer than the strip phase).
-    const bool puller = !MONO || grp < 2;
+    static_assert(sizeof(R) == 8, "FP32 / FP16 storage takes band_tile_mono");
+    const int grp = int(cg::this_cluster().block_rank());
+    const int l = int(threadIdx.x);
     __shared__ __align__(16) R Ys[kTileThreads * 4];        // stage values, lab frame
     __shared__ __align__(16) R Xp[kTileThreads * 8];        // shares of the system's inputs
     __shared__ __align__(16) double Xw[kTileThreads * 4];   // wave amplitudes
@@ -278,86 +581,57 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     R* SNt = SUt1 + 4 * B.max_nodes;               // [max_nodes][5] moments of t
     S* Fx = reinterpret_cast<S*>(SNt + 5 * B.max_nodes);   // [max_fx][Q], node k in CTA k % 4
     auto bcast = [&](auto* p, auto v) {
-        if constexpr (MONO) {
-            *p = v;
-        } else {
-            cg::cluster_group cl = cg::this_cluster();
+        cg::cluster_group cl = cg::this_cluster();
 #pragma unroll
-            for (int q = 0; q < kCluster; ++q) *cl.map_shared_rank(p, q) = v;
-        }
+        for (int q = 0; q < kCluster; ++q) *cl.map_shared_rank(p, q) = v;
     };
-    auto sync_all = [&]() {
-        if constexpr (MONO) __syncthreads();
-        else cg::this_cluster().sync();
-    };
-    // the stage exchanges: a value into slot p of every group, then the wait
+    auto sync_all = [&]() { cg::this_cluster().sync(); };
+    // the stage exchanges: a value into slot p of every CTA, then the wait
     // for all of them
-    auto xput = [&](auto* p, auto v, unsigned long long* bar) {
-        if constexpr (MONO) *p = v;
-        else put_cluster(p, v, bar);
-    };
-    auto xwait = [&](unsigned long long* bar, unsigned parity) -> bool {
-        if constexpr (MONO) {
-            __syncthreads();
-            return true;
-        } else {
-            return wait_exchange(bar, parity, B.status);
-        }
-    };
+    auto xput = [&](auto* p, auto v, unsigned long long* bar) { put_cluster(p, v, bar); };
+    auto xwait = [&](unsigned long long* bar, unsigned parity) -> bool { return wait_exchange(bar, parity, B.status); };
     // Descriptors first, all at once: under a saturated memory system each
     // dependent global round trip costs microseconds.
     const int ns = B.max_nodes;
     const StripNode* snt = B.sn + (long long)tile * ns;
-    // the strip node this thread pulls: node k goes to CTA k % 4 (MONO:
-    // group k % 2), and the nodes of a CTA (group) are dealt round its four
-    // warps
-    constexpr int kPullStride = MONO ? 2 * kTileThreads : kCluster * kTileThreads;
-    const int kp = MONO ? (grp & 1) + 2 * (4 * (l % 32) + l / 32) : grp + kCluster * (4 * (l % 32) + l / 32);
-    // the time-t slots this thread loads: nodes tl, tl + tstride, ...
-    // (descriptors of the first kLT issued here, the rest in a loop); every
-    // CTA of a cluster loads all of them into its own shared memory
+    // the strip node this thread pulls: node k goes to CTA k % 4, and the
+    // nodes of a CTA are dealt round its four warps
+    constexpr int kPullStride = kCluster * kTileThreads;
+    const int kp = grp + kCluster * (4 * (l % 32) + l / 32);
+    // the time-t slots this thread loads: nodes l, l + 128, ... (descriptors
+    // of the first kLT issued here, the rest in a loop); every CTA of a
+    // cluster loads all of them into its own shared memory
     constexpr int kLT = 3;
-    constexpr int tstride = MONO ? 2 * kTileThreads : kTileThreads;
-    const int tl = MONO ? int(threadIdx.x) : l;
-    auto load_desc = [&](StripNode& Nb, int* tsl) {
-        Nb = StripNode{-1, -1, 0, -1, -1, 0};
-        if (puller && kp < ns) Nb = snt[kp];
+    StripNode Nb{-1, -1, 0, -1, -1, 0};
+    int tsl[kLT];
+    if (kp < ns) Nb = snt[kp];
 #pragma unroll
-        for (int j = 0; j < kLT; ++j) {
-            const int k = tl + j * tstride;
-            tsl[j] = -1;
-            if (puller && k < ns) {
-                const StripNode& N = snt[k];
-                if (N.x >= 0 && (N.flags & kSNLoadT)) tsl[j] = N.tslot;
-            }
+    for (int j = 0; j < kLT; ++j) {
+        const int k = l + j * kTileThreads;
+        tsl[j] = -1;
+        if (k < ns) {
+            const StripNode& N = snt[k];
+            if (N.x >= 0 && (N.flags & kSNLoadT)) tsl[j] = N.tslot;
         }
-    };
-    // the cluster form issues them before its cluster barrier; the one-CTA
-    // form at the start of the strip phase (they are dead after it)
-    StripNode NbC;
-    int tslC[kLT];
-    if constexpr (!MONO) load_desc(NbC, tslC);
-    const UDesc D = B.ld[(long long)tile * kTileUnknowns + l];
-    int nc0 = 0, nc1 = 0, nc2 = 0, nc3 = 0;
-    if constexpr (!MONO) {
-        if (l == 0) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&xbar[k])));
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        // unknowns that compute stage s (the same in every CTA of the cluster)
-        nc0 = __syncthreads_count(D.level <= 3);
-        nc1 = __syncthreads_count(D.level <= 2);
-        nc2 = __syncthreads_count(D.level <= 1);
-        nc3 = __syncthreads_count(D.level <= 0);
     }
-    if constexpr (!MONO) sync_all();    // every CTA of the cluster runs before any remote store
+    const UDesc D = B.ld[(long long)tile * kTileUnknowns + l];
+    // the unknown whose populations this thread writes at the end: CTA r
+    // writes unknowns 32 r .. 32 r + 31
+    const UDesc Dw = B.ld[(long long)tile * kTileUnknowns + 32 * grp + l % 32];
+    if (l == 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&xbar[k])));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // unknowns that compute stage s (the same in every CTA of the cluster)
+    const int nc0 = __syncthreads_count(D.level <= 3), nc1 = __syncthreads_count(D.level <= 2),
+              nc2 = __syncthreads_count(D.level <= 1), nc3 = __syncthreads_count(D.level <= 0);
+    sync_all();                         // every CTA of the cluster runs before any remote store
 
     // 1. strip nodes: macros of t and moments of t for every CTA; macros of
-    //    t + 1 (pull and Eq. macro) by CTA k % kCluster (MONO: group k % 2)
-    //    for node k, shared out; post-collision populations of Eq. NEEP
-    //    sources kept locally
+    //    t + 1 (pull and Eq. macro) by CTA k % kCluster for node k, shared out;
+    //    post-collision populations of Eq. NEEP sources kept locally
     const R* gU = static_cast<const R*>(E.stripU) + (long long)par_t * E.nslots * 4;
     const R* gN = static_cast<const R*>(E.stripN) + (long long)par_t * E.nslots * 5;
     const bool meso = B.viscous == VIS_MESO;
@@ -402,25 +676,22 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
             }
         }
     };
-    // U(t) of the tile's unknowns, loaded with the strip's own loads: in the
-    // cluster form by every CTA, which keeps its component grp (u0g); in
-    // the one-CTA form by group 0, which leaves it in shared memory for all
-    // groups (Ys in R, U0s in FP64)
+    // U(t) of the tile's unknowns, loaded with the strip's own loads by every
+    // CTA, which keeps its component grp (u0r)
     const int lev = D.level;            // > 4: no unknown on this thread
-    __shared__ __align__(16) double U0s[MONO ? 4 * kTileThreads : 1];
-    double u0g = 0.0;
-    auto strip = [&](const StripNode& Nb, const int* tsl) {
+    double u0r;
+    {
         double U0[4] = {0.0, 0.0, 0.0, 0.0};
-        if (lev <= 4 && (!MONO || grp == 0)) {
+        if (lev <= 4) {
             const double2* p = reinterpret_cast<const double2*>(B.Ub + ((long long)par_t * B.n_unk + D.gid) * 4);
             const double2 a = p[0], b = p[1];
             U0[0] = a.x; U0[1] = a.y; U0[2] = b.x; U0[3] = b.y;
         }
 #pragma unroll
         for (int j = 0; j < kLT; ++j)
-            if (tsl[j] >= 0) load_t(tl + j * tstride, tsl[j]);
+            if (tsl[j] >= 0) load_t(l + j * kTileThreads, tsl[j]);
         if (Nb.x >= 0 && (Nb.flags & kSNPull)) pull_t1(kp, Nb);
-        for (int k = tl + kLT * tstride; k < ns; k += tstride) {
+        for (int k = l + kLT * kTileThreads; k < ns; k += kTileThreads) {
             const StripNode N = snt[k];
             if (N.x >= 0 && (N.flags & kSNLoadT)) load_t(k, N.tslot);
         }
@@ -428,476 +699,317 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
             const StripNode N = snt[k];
             if (N.x >= 0 && (N.flags & kSNPull)) pull_t1(k, N);
         }
-        if (lev <= 4 && (!MONO || grp == 0)) {
+        if (lev <= 4) {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                Ys[4 * l + m] = R(U0[m]);
-                if constexpr (MONO) U0s[4 * l + m] = U0[m];
+            for (int m = 0; m < 4; ++m) Ys[4 * l + m] = R(U0[m]);
+        }
+        u0r = grp == 0 ? U0[0] : grp == 1 ? U0[1] : grp == 2 ? U0[2] : U0[3];
+    }
+    sync_all();
+
+    // 2. RK4, component grp of every unknown
+    const int rank = grp;
+    CtxT<R> X;
+    X.Y = Ys;
+    X.St = SUt;
+    X.St1 = SUt1;
+    const R rho0r = rho0_of<R>(G), cs2r = R(L::CS2), kr = bconst<R>(B.kR, B.kR_f);
+    const R kAr = bconst<R>(B.kA, B.kA_f), kBr = bconst<R>(B.kB, B.kB_f), ihcsr = bconst<R>(B.ihcs, B.ihcs_f),
+            csr_ = bconst<R>(B.cs, B.cs_f);
+    const bool corner = lev <= 4 && D.kind >= 4;
+    const int scheme = corner ? SCH_LODI : (lev <= 4 ? B.scheme[D.kind] : 0);
+    const bool cbc = scheme == SCH_CBC || scheme == SCH_CBC_RELAX;
+    double acc = 0.0, kc = 0.0;         // lab component rank of sum k and of the last k
+    bool incoming = false;              // wave rank incoming at time t
+    bool xok = true;                    // every exchange so far completed in time
+    for (int stage = 0; stage < 4; ++stage) {
+        const bool comp = lev <= 3 - stage;
+        if (l == 0) {                   // bytes of this stage's two exchanges
+            const unsigned ncomp = unsigned(stage == 0 ? nc0 : stage == 1 ? nc1 : stage == 2 ? nc2 : nc3);
+            expect_bytes(&xbar[stage & 1], unsigned(kCluster * sizeof(double)) * ncomp);
+            expect_bytes(&xbar[2 + (stage & 1)], unsigned(kCluster * sizeof(R)) * ncomp);
+        }
+        X.frac = stage == 0 ? R(0) : (stage == 3 ? R(1) : R(0.5));
+        R Ul[4] = {0, 0, 0, 0}, dUn[4] = {0, 0, 0, 0};
+        R d_ut = 0;
+        // A: inputs of the system, type R: 1/rho, the transversal terms,
+        // sqrt(theta), 1/sqrt(theta), P - P_inf and d(rho T)/dt (thermal) or
+        // d rho/dt (isothermal)
+        if (comp) {
+            const int kind = D.kind;
+            R A[4], Bv[4], Up[4], Um[4];
+            fetch_local(X, l, kind, kr, Ul);
+            if (corner) {
+                // LODI along the outward diagonal, one-sided difference of
+                // spacing sqrt(2) through the two diagonal bulk nodes
+                fetch_local(X, D.nb[0], kind, kr, A);
+                fetch_local(X, D.nb[1], kind, kr, Bv);
+                const R kC = bconst<R>(B.kC, B.kC_f);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) dUn[m] = (R(3) * Ul[m] - R(4) * A[m] + Bv[m]) * kC;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) Up[m] = Um[m] = R(0);
+            } else {
+                if (D.j == B.M) {        // Eq. FD-dx-bw at the outermost layer
+                    fetch_local(X, D.nb[1], kind, kr, A);
+                    fetch_local(X, D.nb[2], kind, kr, Bv);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) dUn[m] = R(0.5) * (R(3) * Ul[m] - R(4) * A[m] + Bv[m]);
+                } else {                 // Eq. FD-dx-center at inner layers
+                    fetch_local(X, D.nb[0], kind, kr, A);
+                    fetch_local(X, D.nb[1], kind, kr, Bv);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) dUn[m] = R(0.5) * (A[m] - Bv[m]);
+                }
+                fetch_local(X, D.nb[4], kind, kr, Up);
+                fetch_local(X, D.nb[5], kind, kr, Um);
+            }
+            d_ut = R(0.5) * (Up[2] - Um[2]);
+            // share q of the inputs (q = 0..3: entries {0,1}, {2,3},
+            // {4,5,6 isothermal}, {6,7 thermal})
+            auto input = [&](int i) -> R {
+                switch (i) {
+                case 0: return R(1) / (rho0r + Ul[0]);
+                case 1: return corner ? R(0) : R(-0.5) * ((rho0r + Up[0]) * Up[2] - (rho0r + Um[0]) * Um[2]);
+                case 2: return TH ? sqrt_r(R(1) + Ul[3]) : R(0);
+                case 3: return corner ? R(0) : -Ul[2] * (R(0.5) * (Up[1] - Um[1]));
+                case 4: return TH ? rsqrt_r(R(1) + Ul[3]) : R(0);
+                case 5: {
+                    const R dP = TH ? cs2r * (Ul[0] + rho0r * Ul[3] + Ul[0] * Ul[3]) : cs2r * Ul[0];
+                    return corner ? R(0) : dP - bconst<R>(B.pdev[kind], B.pdev_f[kind]);
+                }
+                case 6:
+                    // rho T - rho0 = drho + rho0 dT + drho dT
+                    return TH ? R(0.5) * ((Up[0] + rho0r * Up[3] + Up[0] * Up[3]) -
+                                          (Um[0] + rho0r * Um[3] + Um[0] * Um[3]))
+                              : R(0.5) * (Up[0] - Um[0]);
+                default:
+                    return (TH && !corner) ? R(-0.5) * ((R(1) + Up[3]) * Up[2] - (R(1) + Um[3]) * Um[2]) : R(0);
+                }
+            };
+            R* xp = Xp + 8 * l;
+            if (rank == 0) {
+                bcast(xp + 0, input(0));
+                bcast(xp + 1, input(1));
+            } else if (rank == 1) {
+                if (TH) bcast(xp + 2, input(2));
+                bcast(xp + 3, input(3));
+            } else if (rank == 2) {
+                if (TH) bcast(xp + 4, input(4));
+                bcast(xp + 5, input(5));
+                if (!TH) bcast(xp + 6, input(6));
+            } else if (TH) {
+                bcast(xp + 6, input(6));
+                bcast(xp + 7, input(7));
+            }
+            if (stage == 0) {
+                R v = R(0);
+                if (!corner && B.viscous == VIS_FD) v = vis_fd_c<TH, R>(rank, G, B, X, D, l, cs2r);
+                else if (!corner && B.viscous == VIS_MESO) v = vis_meso_c<TH, R>(rank, G, SUt, SNt, D, cs2r);
+                bcast(Xv + 4 * l + rank, v);
             }
         }
-        if constexpr (!MONO) u0g = grp == 0 ? U0[0] : grp == 1 ? U0[1] : grp == 2 ? U0[2] : U0[3];
-    };
-    if constexpr (!MONO) {
-        strip(NbC, tslC);
         sync_all();
-    }
-
-    // 2. RK4, component rank of every unknown, and 3. the Dirichlet write
-    // (pass 1).  MONO: pass 0 is the strip phase in groups 0 and 1 and the
-    // warm-up in groups 2 and 3, which runs the one copy of this code.
-    static_assert(!MONO || sizeof(R) == 4, "the one-CTA form keeps every input local");
-#pragma unroll 1
-    for (int pass = MONO ? 0 : 1; pass < 2; ++pass) {
-      const bool dry = pass == 0;
-      if (dry && puller) {
-        StripNode Nb;
-        int tsl[kLT];
-        load_desc(Nb, tsl);
-        strip(Nb, tsl);
-      } else {
-        // warm-up: eight warps, one code part each (0: A's stencils and
-        // inputs, 1: A's viscous vector, 2: B, 3 and 4: C in roles 0-1 and
-        // 2-3, 5: the Dirichlet write, 6 and 7: none) with their lanes in
-        // every role of the part; the real pass: part 8, all of it
-        const int part = dry ? int(threadIdx.x / 32) % 8 : 8;
-        const int rank = !dry ? grp
-                       : part == 3 ? int(threadIdx.x % 2)
-                       : part == 4 ? 2 + int(threadIdx.x % 2) : int(threadIdx.x % 4);
-        CtxT<R> X;
-        X.Y = Ys;
-        X.St = SUt;
-        X.St1 = SUt1;
-        const R rho0r = rho0_of<R>(G), cs2r = R(L::CS2), kr = bconst<R>(B.kR, B.kR_f);
-        const R kAr = bconst<R>(B.kA, B.kA_f), kBr = bconst<R>(B.kB, B.kB_f), ihcsr = bconst<R>(B.ihcs, B.ihcs_f),
-                csr_ = bconst<R>(B.cs, B.cs_f);
-        const bool corner = lev <= 4 && D.kind >= 4;
-        const int scheme = corner ? SCH_LODI : (lev <= 4 ? B.scheme[D.kind] : 0);
-        const bool cbc = scheme == SCH_CBC || scheme == SCH_CBC_RELAX;
-        double acc = 0.0, kc = 0.0;         // lab component rank of sum k and of the last k
-        const double u0r = [&] {            // component grp of U(t)
-            if constexpr (MONO) return U0s[4 * l + grp];
-            else return u0g;
-        }();
-        FF accf{0.0f, 0.0f};                // the same sum in float-float (FP32 / FP16 storage)
-        const FF u0f = ff_split(u0r);
-        bool incoming = false;              // wave rank incoming at time t
-        // In FP32 every CTA forms all inputs of the system itself; in FP64 each
-        // CTA forms a share and the shares are exchanged (FP64 issue is slow).
-        constexpr bool kLocal = sizeof(R) == 4;
-        R xs[8] = {0, 0, 0, 0, 0, 0, 0, 0}; // the inputs, kLocal
-        R Vs[4] = {0, 0, 0, 0};             // viscous vector (local frame, frozen), kLocal
-        bool xok = true;                    // every exchange so far completed in time
-        for (int stage = 0; stage < (dry ? 1 : 4); ++stage) {
-            const bool comp = lev <= 3 - stage;
-            if (!MONO && l == 0) {          // bytes of this stage's two exchanges
-                const unsigned ncomp = unsigned(stage == 0 ? nc0 : stage == 1 ? nc1 : stage == 2 ? nc2 : nc3);
-                expect_bytes(&xbar[stage & 1], unsigned(kCluster * sizeof(double)) * ncomp);
-                expect_bytes(&xbar[2 + (stage & 1)], unsigned(kCluster * sizeof(R)) * ncomp);
+        // B: wave rank, FP64.  Row rank of S (see apply_S) applied to dU/dn,
+        // T and V, with Lambda_rank.
+        auto XP = [&](int i) -> R { return Xp[8 * l + i]; };
+        R TTr[4] = {0, 0, 0, 0};        // transversal terms, local frame
+        R Vr[4] = {0, 0, 0, 0};
+        if (comp) {
+            if (!corner) {
+                TTr[0] = XP(1);
+                TTr[1] = XP(3);
+                TTr[2] = -cs2r * XP(0) * XP(6) - Ul[2] * d_ut;
+                TTr[3] = TH ? XP(7) : R(0);
             }
-            X.frac = stage == 0 ? R(0) : (stage == 3 ? R(1) : R(0.5));
-            R Ul[4] = {0, 0, 0, 0}, dUn[4] = {0, 0, 0, 0};
-            R d_ut = 0;
-            // A: inputs of the system, type R: 1/rho, the transversal terms,
-            // sqrt(theta), 1/sqrt(theta), P - P_inf and d(rho T)/dt (thermal) or
-            // d rho/dt (isothermal)
-            if (comp && (part == 8 || part <= 1)) {
-                const int kind = D.kind;
-                R A[4], Bv[4], Up[4], Um[4];
-                if (part != 1) {             // (the warm-up's part 1: the viscous vector only)
-                    fetch_local(X, l, kind, kr, Ul);
-                    if (corner) {
-                        // LODI along the outward diagonal, one-sided difference of
-                        // spacing sqrt(2) through the two diagonal bulk nodes
-                        fetch_local(X, D.nb[0], kind, kr, A);
-                        fetch_local(X, D.nb[1], kind, kr, Bv);
-                        const R kC = bconst<R>(B.kC, B.kC_f);
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) dUn[m] = (R(3) * Ul[m] - R(4) * A[m] + Bv[m]) * kC;
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) Up[m] = Um[m] = R(0);
-                    } else {
-                        if (D.j == B.M) {        // Eq. FD-dx-bw at the outermost layer
-                            fetch_local(X, D.nb[1], kind, kr, A);
-                            fetch_local(X, D.nb[2], kind, kr, Bv);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) dUn[m] = R(0.5) * (R(3) * Ul[m] - R(4) * A[m] + Bv[m]);
-                        } else {                 // Eq. FD-dx-center at inner layers
-                            fetch_local(X, D.nb[0], kind, kr, A);
-                            fetch_local(X, D.nb[1], kind, kr, Bv);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) dUn[m] = R(0.5) * (A[m] - Bv[m]);
-                        }
-                        fetch_local(X, D.nb[4], kind, kr, Up);
-                        fetch_local(X, D.nb[5], kind, kr, Um);
-                    }
-                    d_ut = R(0.5) * (Up[2] - Um[2]);
-                }
-                // share q of the inputs (q = 0..3: entries {0,1}, {2,3},
-                // {4,5,6 isothermal}, {6,7 thermal})
-                auto input = [&](int i) -> R {
-                    switch (i) {
-                    case 0: return R(1) / (rho0r + Ul[0]);
-                    case 1: return corner ? R(0) : R(-0.5) * ((rho0r + Up[0]) * Up[2] - (rho0r + Um[0]) * Um[2]);
-                    case 2: return TH ? sqrt_r(R(1) + Ul[3]) : R(0);
-                    case 3: return corner ? R(0) : -Ul[2] * (R(0.5) * (Up[1] - Um[1]));
-                    case 4: return TH ? rsqrt_r(R(1) + Ul[3]) : R(0);
-                    case 5: {
-                        const R dP = TH ? cs2r * (Ul[0] + rho0r * Ul[3] + Ul[0] * Ul[3]) : cs2r * Ul[0];
-                        return corner ? R(0) : dP - bconst<R>(B.pdev[kind], B.pdev_f[kind]);
-                    }
-                    case 6:
-                        // rho T - rho0 = drho + rho0 dT + drho dT
-                        return TH ? R(0.5) * ((Up[0] + rho0r * Up[3] + Up[0] * Up[3]) -
-                                              (Um[0] + rho0r * Um[3] + Um[0] * Um[3]))
-                                  : R(0.5) * (Up[0] - Um[0]);
-                    default:
-                        return (TH && !corner) ? R(-0.5) * ((R(1) + Up[3]) * Up[2] - (R(1) + Um[3]) * Um[2]) : R(0);
-                    }
-                };
-                if constexpr (kLocal) {
-                    if (part != 1) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) xs[i] = input(i);
-                    }
-                    if (stage == 0 && !corner && part != 0) {
-                        if (B.viscous == VIS_FD) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) Vs[c] = vis_fd_c<TH, R>(c, G, B, X, D, l, cs2r);
-                        } else if (B.viscous == VIS_MESO) {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) Vs[c] = vis_meso_c<TH, R>(c, G, SUt, SNt, D, cs2r);
-                        }
-                    }
-                } else {
-                    R* xp = Xp + 8 * l;
-                    if (rank == 0) {
-                        bcast(xp + 0, input(0));
-                        bcast(xp + 1, input(1));
-                    } else if (rank == 1) {
-                        if (TH) bcast(xp + 2, input(2));
-                        bcast(xp + 3, input(3));
-                    } else if (rank == 2) {
-                        if (TH) bcast(xp + 4, input(4));
-                        bcast(xp + 5, input(5));
-                        if (!TH) bcast(xp + 6, input(6));
-                    } else if (TH) {
-                        bcast(xp + 6, input(6));
-                        bcast(xp + 7, input(7));
-                    }
-                    if (stage == 0) {
-                        R v = R(0);
-                        if (!corner && B.viscous == VIS_FD) v = vis_fd_c<TH, R>(rank, G, B, X, D, l, cs2r);
-                        else if (!corner && B.viscous == VIS_MESO) v = vis_meso_c<TH, R>(rank, G, SUt, SNt, D, cs2r);
-                        bcast(Xv + 4 * l + rank, v);
-                    }
-                }
-            }
-            if constexpr (!kLocal) sync_all();
-            // B: wave rank, FP64.  Row rank of S (see apply_S) applied to dU/dn,
-            // T and V, with Lambda_rank.
-            auto XP = [&](int i) -> R {
-                if constexpr (kLocal) return xs[i];
-                else return Xp[8 * l + i];
-            };
-            R TTr[4] = {0, 0, 0, 0};        // transversal terms, local frame
-            R Vr[4] = {0, 0, 0, 0};
-            if (comp && (part == 8 || part == 2)) {
-                if (!corner) {
-                    TTr[0] = XP(1);
-                    TTr[1] = XP(3);
-                    TTr[2] = -cs2r * XP(0) * XP(6) - Ul[2] * d_ut;
-                    TTr[3] = TH ? XP(7) : R(0);
-                }
-                if constexpr (kLocal) {
-                    Vr[1] = Vs[1];
-                    Vr[2] = Vs[2];
-                    Vr[3] = TH ? Vs[0] + Vs[3] : R(0);      // V0 = 0; V3 from two shares
-                } else {
-                    const R* xv = Xv + 4 * l;
-                    Vr[1] = xv[1];
-                    Vr[2] = xv[2];
-                    Vr[3] = TH ? xv[0] + xv[3] : R(0);
-                }
-                // Row `rank` of S (see apply_S) and Lambda_rank.  Their entries
-                // are formed from the inputs in type R (the inputs' own
-                // precision) and only the non-zero ones enter the FP64
-                // projections: thermal rows (-r/2, 0, 0, 1/2), (0, 0, 1, 0),
-                // (r/4, -+a, 0, 1/4); isothermal rows (1/2, -+h, 0), (0, 0, 1).
-                R c0 = R(0), c1 = R(0), c3 = R(0), lamr = Ul[1];
-                bool acoustic = false;
-                if (TH) {
-                    const R rr = (R(1) + Ul[3]) * XP(0);
-                    if (rank == 0) {
-                        c0 = R(-0.5) * rr;
-                        c3 = R(0.5);
-                    } else if (rank >= 2) {
-                        const R sg = rank == 2 ? R(-1) : R(1);
-                        c0 = R(0.25) * rr;
-                        c1 = sg * XP(2) * kAr;
-                        c3 = R(0.25);
-                        lamr = Ul[1] + sg * XP(2) * kBr;
-                        acoustic = true;
-                    }
-                } else if (rank == 0 || rank == 2) {
-                    const R sg = rank == 0 ? R(-1) : R(1);
-                    c0 = R(0.5);
-                    c1 = sg * (rho0r + Ul[0]) * ihcsr;
-                    lamr = Ul[1] + sg * csr_;
+            const R* xv = Xv + 4 * l;
+            Vr[1] = xv[1];
+            Vr[2] = xv[2];
+            Vr[3] = TH ? xv[0] + xv[3] : R(0);
+            // Row `rank` of S (see apply_S) and Lambda_rank.  Their entries
+            // are formed from the inputs in type R (the inputs' own
+            // precision) and only the non-zero ones enter the FP64
+            // projections: thermal rows (-r/2, 0, 0, 1/2), (0, 0, 1, 0),
+            // (r/4, -+a, 0, 1/4); isothermal rows (1/2, -+h, 0), (0, 0, 1).
+            R c0 = R(0), c1 = R(0), c3 = R(0), lamr = Ul[1];
+            bool acoustic = false;
+            if (TH) {
+                const R rr = (R(1) + Ul[3]) * XP(0);
+                if (rank == 0) {
+                    c0 = R(-0.5) * rr;
+                    c3 = R(0.5);
+                } else if (rank >= 2) {
+                    const R sg = rank == 2 ? R(-1) : R(1);
+                    c0 = R(0.25) * rr;
+                    c1 = sg * XP(2) * kAr;
+                    c3 = R(0.25);
+                    lamr = Ul[1] + sg * XP(2) * kBr;
                     acoustic = true;
                 }
-                double w = 0.0;
-                if constexpr (kLocal) {
-                    // the wave in float-float; every product of two inputs is
-                    // exact in it, as in FP64
-                    auto srow = [&](const R* v) -> FF {
-                        if (rank == 1) return FF{v[2], 0.0f};
-                        if (TH) {
-                            const FF sr = ff_add(ff_prod(c0, v[0]), ff_prod(c3, v[3]));
-                            return rank == 0 ? sr : ff_add(sr, ff_prod(c1, v[1]));
-                        }
-                        return ff_add(ff_prod(c0, v[0]), ff_prod(c1, v[1]));
-                    };
-                    if (stage == 0) incoming = lamr < R(0);
-                    FF wf{0.0f, 0.0f};
-                    if (TH || rank != 3) {
-                        if (!incoming) {
-                            wf = ff_mul(srow(dUn), lamr);
-                        } else if (scheme != SCH_LODI) {
-                            const FF st = srow(TTr);
-                            const FF relaxP = acoustic ? ff_mul(ff_const(B.ffk[FFK_BP]), XP(5)) : FF{0.0f, 0.0f};
-                            if (scheme == SCH_LODI_RELAX) {
-                                wf = ff_add(ff_mul(ff_add(ff_const(B.ffk[FFK_TINF]), ff_neg(st)),
-                                                   ff_const(B.ffk[FFK_AT])),
-                                            relaxP);
-                            } else if (scheme == SCH_CBC) {
-                                wf = B.viscous != VIS_OFF ? ff_add(st, srow(Vr)) : st;
-                            } else {
-                                // Eq. CBC-Relax; the viscous term relaxed towards 0
-                                // at rate alpha_V (0: the paper's equation)
-                                wf = ff_add(ff_mul(st, ff_const(B.ffk[FFK_1MAT])), ff_const(B.ffk[FFK_ATTI]));
-                                if (B.viscous != VIS_OFF) wf = ff_add(wf, ff_mul(srow(Vr), ff_const(B.ffk[FFK_1MAV])));
-                                wf = ff_add(wf, relaxP);
-                            }
-                        }
-                    }
-                    w = ff_pack(wf);
-                } else {
-                    const double d0 = double(c0), d1 = double(c1), d3 = double(c3);
-                    auto srow = [&](const R* v) -> double {
-                        if (rank == 1) return double(v[2]);
-                        if (TH) {
-                            const double sr = d0 * double(v[0]) + d3 * double(v[3]);
-                            return rank == 0 ? sr : sr + d1 * double(v[1]);
-                        }
-                        return d0 * double(v[0]) + d1 * double(v[1]);
-                    };
-                    const double lam = double(lamr);
-                    if (stage == 0) incoming = lam < 0.0;
-                    if (TH || rank != 3) {
-                        if (!incoming) {
-                            w = lam * srow(dUn);
-                        } else if (scheme != SCH_LODI) {
-                            const double st = srow(TTr);
-                            const double relaxP = acoustic ? B.beta_P * double(XP(5)) : 0.0;
-                            if (scheme == SCH_LODI_RELAX) w = B.alpha_T * (B.t_inf - st) + relaxP;
-                            // the viscous projection (none when the viscous vector is off)
-                            else if (scheme == SCH_CBC) w = st + (B.viscous != VIS_OFF ? srow(Vr) : 0.0);
-                            else {
-                                // Eq. CBC-Relax; the viscous term relaxed towards 0
-                                // at rate alpha_V (0: the paper's equation)
-                                const double sv = B.viscous != VIS_OFF ? srow(Vr) : 0.0;
-                                w = (1.0 - B.alpha_T) * st + (1.0 - B.alpha_V) * sv + B.alpha_T * B.t_inf + relaxP;
-                            }
-                        }
-                    }
+            } else if (rank == 0 || rank == 2) {
+                const R sg = rank == 0 ? R(-1) : R(1);
+                c0 = R(0.5);
+                c1 = sg * (rho0r + Ul[0]) * ihcsr;
+                lamr = Ul[1] + sg * csr_;
+                acoustic = true;
+            }
+            double w = 0.0;
+            const double d0 = double(c0), d1 = double(c1), d3 = double(c3);
+            auto srow = [&](const R* v) -> double {
+                if (rank == 1) return double(v[2]);
+                if (TH) {
+                    const double sr = d0 * double(v[0]) + d3 * double(v[3]);
+                    return rank == 0 ? sr : sr + d1 * double(v[1]);
                 }
-                if (!dry) xput(Xw + 4 * l + rank, w, &xbar[stage & 1]);
-                // the transversal and viscous terms this CTA adds in step C
-                if (cbc) {
-                    if (rank == 3) {
-                        TTr[3] += Vr[3];
-                    } else if (rank != 0) {         // V0 = 0
-                        TTr[1] += Vr[1];
-                        TTr[2] += Vr[2];
+                return d0 * double(v[0]) + d1 * double(v[1]);
+            };
+            const double lam = double(lamr);
+            if (stage == 0) incoming = lam < 0.0;
+            if (TH || rank != 3) {
+                if (!incoming) {
+                    w = lam * srow(dUn);
+                } else if (scheme != SCH_LODI) {
+                    const double st = srow(TTr);
+                    const double relaxP = acoustic ? B.beta_P * double(XP(5)) : 0.0;
+                    if (scheme == SCH_LODI_RELAX) w = B.alpha_T * (B.t_inf - st) + relaxP;
+                    // the viscous projection (none when the viscous vector is off)
+                    else if (scheme == SCH_CBC) w = st + (B.viscous != VIS_OFF ? srow(Vr) : 0.0);
+                    else {
+                        // Eq. CBC-Relax; the viscous term relaxed towards 0
+                        // at rate alpha_V (0: the paper's equation)
+                        const double sv = B.viscous != VIS_OFF ? srow(Vr) : 0.0;
+                        w = (1.0 - B.alpha_T) * st + (1.0 - B.alpha_V) * sv + B.alpha_T * B.t_inf + relaxP;
                     }
                 }
             }
-            if (xok && !dry) xok = xwait(&xbar[stage & 1], (stage >> 1) & 1);
-            // C: lab component rank of the right-hand side (S^-1 of the waves,
-            // with r^-1 = rho / theta, b = sqrt(2 c_s^4 / T~) formed in type R);
-            // RK4 update (FP64).  A side unknown's lab component 1 or 2 needs
-            // one local component only.
-            if (comp && (part == 8 || part == 3 || part == 4)) {
-                if constexpr (kLocal) {
-                    // float-float from the waves to the lab component; one
-                    // conversion to FP64 for the RK4 sum
-                    const double* wp = Xw + 4 * l;
-                    const FF w0 = ff_unpack(wp[0]), w1 = ff_unpack(wp[1]), w2 = ff_unpack(wp[2]),
-                             w3 = ff_unpack(wp[3]);
-                    const FF zero{0.0f, 0.0f};
-                    FF kl1 = zero, kl2 = zero, klr = zero;
-                    if (rank == 0) {
-                        if (TH) {
-                            const R irr = (rho0r + Ul[0]) * XP(4) * XP(4);
-                            klr = ff_neg(ff_mul(ff_add(ff_add(w2, w3), ff_neg(w0)), irr));
-                        } else {
-                            klr = ff_neg(ff_add(w0, w2));
-                        }
-                        if (cbc) klr = ff_add(klr, FF{TTr[0], 0.0f});
-                    } else if (rank == 3) {
-                        klr = TH ? ff_neg(ff_add(ff_add(w0, w2), w3)) : zero;
-                        if (cbc && TH) klr = ff_add(klr, FF{TTr[3], 0.0f});
-                    } else {
-                        const bool sideW = D.kind < 2;
-                        const bool need1 = corner || ((rank == 1) == sideW);
-                        const bool need2 = corner || ((rank == 1) != sideW);
-                        if (need1) {
-                            const R bf = TH ? XP(4) * kBr : csr_ * XP(0);
-                            kl1 = ff_neg(ff_mul(TH ? ff_add(w3, ff_neg(w2)) : ff_add(w2, ff_neg(w0)), bf));
-                            if (cbc) kl1 = ff_add(kl1, FF{TTr[1], 0.0f});
-                        }
-                        if (need2) {
-                            kl2 = ff_neg(w1);
-                            if (cbc) kl2 = ff_add(kl2, FF{TTr[2], 0.0f});
-                        }
-                    }
-                    // lab component (lab_component's selection, in float-float)
-                    FF kf;
-                    if (rank == 0 || rank == 3) {
-                        kf = klr;
-                    } else if (D.kind < 4) {
-                        const int kind = D.kind;
-                        kf = kind == 0 ? (rank == 1 ? ff_neg(kl1) : kl2)
-                           : kind == 1 ? (rank == 1 ? kl1 : kl2)
-                           : kind == 2 ? (rank == 1 ? kl2 : ff_neg(kl1))
-                                       : (rank == 1 ? kl2 : kl1);
-                    } else {
-                        const int c = D.kind - 4;
-                        const FF r = ff_const(B.ffk[FFK_KR]);
-                        const FF n0 = (c & 1) ? r : ff_neg(r), n1 = (c & 2) ? r : ff_neg(r);
-                        kf = rank == 1 ? ff_add(ff_mul(kl1, n0), ff_neg(ff_mul(kl2, n1)))
-                                       : ff_add(ff_mul(kl1, n1), ff_mul(kl2, n0));
-                    }
-                    // RK4 (sum and stage value) in float-float as well: no
-                    // FP64 instruction in the stage loop
-                    if (stage < 3) {
-                        const FF k2 = stage == 0 ? kf : ff_scale(kf, 2.0f);
-                        accf = stage == 0 ? k2 : ff_add(accf, k2);
-                        const FF y = ff_add(u0f, ff_scale(kf, stage == 2 ? 1.0f : 0.5f));
-                        if (!dry) xput(Ys + 4 * l + rank, y.h, &xbar[2 + (stage & 1)]);
-                    } else {
-                        // RK4: U(t + 1) = U(t) + (k1 + 2 k2 + 2 k3 + k4) / 6
-                        const FF un = ff_add(u0f, ff_mul(ff_add(accf, kf), ff_const(B.ffk[FFK_SIXTH])));
-                        if (!dry) {
-                            B.Ub[((long long)(par_t ^ 1) * B.n_unk + D.gid) * 4 + rank] = ff_to_double(un);
-                            xput(Ys + 4 * l + rank, un.h, &xbar[2 + (stage & 1)]);
-                        }
-                    }
-                } else {
-                    const double* w = Xw + 4 * l;
-                    double kl1 = 0.0, kl2 = 0.0, klr = 0.0;
-                    if (rank == 0) {
-                        if (TH) {
-                            const R irr = (rho0r + Ul[0]) * XP(4) * XP(4);
-                            klr = -((w[2] + w[3] - w[0]) * double(irr));
-                        } else {
-                            klr = -(w[0] + w[2]);
-                        }
-                        if (cbc) klr += double(TTr[0]);
-                    } else if (rank == 3) {
-                        klr = TH ? -(w[0] + w[2] + w[3]) : 0.0;
-                        if (cbc && TH) klr += double(TTr[3]);
-                    } else {
-                        const bool sideW = D.kind < 2;
-                        const bool need1 = corner || ((rank == 1) == sideW);
-                        const bool need2 = corner || ((rank == 1) != sideW);
-                        if (need1) {
-                            const R bf = TH ? XP(4) * kBr : csr_ * XP(0);
-                            kl1 = -(double(bf) * (TH ? w[3] - w[2] : w[2] - w[0]));
-                            if (cbc) kl1 += double(TTr[1]);
-                        }
-                        if (need2) {
-                            kl2 = -w[1];
-                            if (cbc) kl2 += double(TTr[2]);
-                        }
-                    }
-                    kc = lab_component(rank, D.kind, B.kR, klr, kl1, kl2, klr);
-                    if (stage < 3) {
-                        const double wk = stage == 0 ? 1.0 : 2.0;
-                        const double hk = stage == 2 ? 1.0 : 0.5;
-                        acc = (stage == 0 ? 0.0 : acc) + wk * kc;
-                        if (!dry) xput(Ys + 4 * l + rank, R(u0r + hk * kc), &xbar[2 + (stage & 1)]);
-                    } else {
-                        // RK4: U(t + 1) = U(t) + (k1 + 2 k2 + 2 k3 + k4) / 6
-                        const double un = u0r + (acc + kc) * (1.0 / 6.0);
-                        if (!dry) {
-                            B.Ub[((long long)(par_t ^ 1) * B.n_unk + D.gid) * 4 + rank] = un;
-                            xput(Ys + 4 * l + rank, R(un), &xbar[2 + (stage & 1)]);
-                        }
-                    }
+            xput(Xw + 4 * l + rank, w, &xbar[stage & 1]);
+            // the transversal and viscous terms this CTA adds in step C
+            if (cbc) {
+                if (rank == 3) {
+                    TTr[3] += Vr[3];
+                } else if (rank != 0) {         // V0 = 0
+                    TTr[1] += Vr[1];
+                    TTr[2] += Vr[2];
                 }
             }
-            if (xok && !dry) xok = xwait(&xbar[2 + (stage & 1)], (stage >> 1) & 1);
         }
-
-        // 3. Dirichlet populations of unknown l, on CTA l % kCluster
-        if (lev == 0 && l % kCluster == rank && (part == 8 || part == 5)) {
-            const R Unew[4] = {Ys[4 * l], Ys[4 * l + 1], Ys[4 * l + 2], Ys[4 * l + 3]};
-            const bool neep = B.dirichlet >= 1;     // needs x_f: NEEP or regularised NEEP
-            const S* fs = nullptr;
-            if (neep) {
-                if constexpr (MONO) fs = Fx + D.wsrc * L::Q;
-                else fs = cg::this_cluster().map_shared_rank(Fx + D.wsrc * L::Q, D.wslot % kCluster);
+        if (xok) xok = xwait(&xbar[stage & 1], (stage >> 1) & 1);
+        // C: lab component rank of the right-hand side (S^-1 of the waves,
+        // with r^-1 = rho / theta, b = sqrt(2 c_s^4 / T~) formed in type R);
+        // RK4 update (FP64).  A side unknown's lab component 1 or 2 needs
+        // one local component only.
+        if (comp) {
+            const double* w = Xw + 4 * l;
+            double kl1 = 0.0, kl2 = 0.0, klr = 0.0;
+            if (rank == 0) {
+                if (TH) {
+                    const R irr = (rho0r + Ul[0]) * XP(4) * XP(4);
+                    klr = -((w[2] + w[3] - w[0]) * double(irr));
+                } else {
+                    klr = -(w[0] + w[2]);
+                }
+                if (cbc) klr += double(TTr[0]);
+            } else if (rank == 3) {
+                klr = TH ? -(w[0] + w[2] + w[3]) : 0.0;
+                if (cbc && TH) klr += double(TTr[3]);
+            } else {
+                const bool sideW = D.kind < 2;
+                const bool need1 = corner || ((rank == 1) == sideW);
+                const bool need2 = corner || ((rank == 1) != sideW);
+                if (need1) {
+                    const R bf = TH ? XP(4) * kBr : csr_ * XP(0);
+                    kl1 = -(double(bf) * (TH ? w[3] - w[2] : w[2] - w[0]));
+                    if (cbc) kl1 += double(TTr[1]);
+                }
+                if (need2) {
+                    kl2 = -w[1];
+                    if (cbc) kl2 += double(TTr[2]);
+                }
             }
-            dirichlet<LAT, S, R, REF>(G, B, f, neep ? SUt1 + 4 * D.wslot : nullptr, fs, D, Unew, dry);
+            kc = lab_component(rank, D.kind, B.kR, klr, kl1, kl2, klr);
+            if (stage < 3) {
+                const double wk = stage == 0 ? 1.0 : 2.0;
+                const double hk = stage == 2 ? 1.0 : 0.5;
+                acc = (stage == 0 ? 0.0 : acc) + wk * kc;
+                xput(Ys + 4 * l + rank, R(u0r + hk * kc), &xbar[2 + (stage & 1)]);
+            } else {
+                // RK4: U(t + 1) = U(t) + (k1 + 2 k2 + 2 k3 + k4) / 6
+                const double un = u0r + (acc + kc) * (1.0 / 6.0);
+                B.Ub[((long long)(par_t ^ 1) * B.n_unk + D.gid) * 4 + rank] = un;
+                xput(Ys + 4 * l + rank, R(un), &xbar[2 + (stage & 1)]);
+            }
         }
-      }
-      if (dry) sync_all();              // the strip phase (and the warm-up) are complete
+        if (xok) xok = xwait(&xbar[2 + (stage & 1)], (stage >> 1) & 1);
     }
-    if constexpr (!MONO) cg::this_cluster().sync();   // no CTA leaves while its Fx may be read
+
+    // 3. Dirichlet populations of unknown Dw: each of the CTA's four warps a
+    // quarter of the velocity pairs (one warp instruction of FP64 costs 64
+    // cycles however few lanes are active, so all lanes of four
+    // sub-partitions share the equilibrium's 200 to 450 of them)
+    if (Dw.level == 0) {
+        const int u = 32 * grp + l % 32;
+        const R Unew[4] = {Ys[4 * u], Ys[4 * u + 1], Ys[4 * u + 2], Ys[4 * u + 3]};
+        const bool neep = B.dirichlet >= 1;     // needs x_f: NEEP or regularised NEEP
+        const S* fs = neep ? cg::this_cluster().map_shared_rank(Fx + Dw.wsrc * L::Q, Dw.wslot % kCluster) : nullptr;
+        const R* us = neep ? SUt1 + 4 * Dw.wslot : nullptr;
+        switch (l / 32) {
+        case 0: dirichlet<LAT, S, R, REF, 0, 4>(G, B, f, us, fs, Dw, Unew); break;
+        case 1: dirichlet<LAT, S, R, REF, 1, 4>(G, B, f, us, fs, Dw, Unew); break;
+        case 2: dirichlet<LAT, S, R, REF, 2, 4>(G, B, f, us, fs, Dw, Unew); break;
+        default: dirichlet<LAT, S, R, REF, 3, 4>(G, B, f, us, fs, Dw, Unew);
+        }
+    }
+    cg::this_cluster().sync();          // no CTA leaves while its Fx may be read
 }
 
-// The tile form by storage.  FP32 / FP16: one 512-thread CTA per tile, at
-// most 128 registers a thread (the whole register file of its SM, which
-// then holds no bulk CTA: the bulk kernel runs undisturbed on the other
-// SMs).  FP64: a cluster of four 128-thread CTAs (launched with the cluster
-// attribute), its FP64 wave arithmetic spread over four SMs.
+// The tile form by storage.  FP32 / FP16: one CTA per tile (band_tile_mono),
+// 512 threads of at most 128 registers in a grid's own launch (the whole
+// register file of its SM, which then holds no bulk CTA: the bulk kernel
+// runs undisturbed on the other SMs).  FP64: a cluster of four 128-thread
+// CTAs (launched with the cluster attribute), its FP64 wave arithmetic
+// spread over four SMs.
 template <typename S>
 constexpr bool band_mono() { return sizeof(S) < 8; }
+template <typename S>
+constexpr int band_threads() { return band_mono<S>() ? 4 * kTileThreads : kTileThreads; }
 
-template <int LAT, typename S, bool REF, bool MONO>
-__global__ void __launch_bounds__(band_threads<MONO>(), 1)
+template <int LAT, typename S, bool REF>
+__global__ void __launch_bounds__(band_threads<S>(), 1)
     k_band(Geom G, Offsets O, Band B, Export E, const S* __restrict__ fin, S* __restrict__ f,
            int par_t)
 {
-    if constexpr (MONO) {
+    if constexpr (band_mono<S>()) {
         for (int t = blockIdx.x; t < B.n_tiles; t += gridDim.x) {
-            band_tile<LAT, S, REF, MONO>(G, O, B, E, fin, f, par_t, t);
+            band_tile_mono<LAT, S, REF, true>(G, O, B, E, fin, f, par_t, t);
             __syncthreads();            // the next tile reuses the shared memory
         }
     } else {
-        band_tile<LAT, S, REF, MONO>(G, O, B, E, fin, f, par_t, blockIdx.x / kCluster);
+        band_tile<LAT, S, REF>(G, O, B, E, fin, f, par_t, blockIdx.x / kCluster);
     }
 }
 
 // Band tiles of many grids in one launch: CTA (cluster) t takes tile
 // tile_run[t].y of run tile_run[t].x, whose structures it copies to shared
-// memory first; the tile form as in k_band.
+// memory first.  FP32 / FP16: 128 threads per tile, four CTAs resident per
+// SM (a tile holds no SM alone, so one tile's round trips and barriers run
+// beside the others' arithmetic; 1806 D2Q37 tiles took 259 us with one
+// 512-thread CTA per SM, now 153 us, 600 D2Q9 tiles 79 us, now 40 us).
 template <int LAT, typename S>
-__global__ void __launch_bounds__(band_threads<band_mono<S>()>(), 1)
+__global__ void __launch_bounds__(kTileThreads, band_mono<S>() ? 4 : 1)
     k_band_batch(const BandRun* __restrict__ runs, const int2* __restrict__ tile_run, int par_t)
 {
-    constexpr bool MONO = band_mono<S>();
     __shared__ __align__(16) BandRun R;
-    const int2 tr = tile_run[MONO ? blockIdx.x : blockIdx.x / kCluster];
+    const int2 tr = tile_run[band_mono<S>() ? blockIdx.x : blockIdx.x / kCluster];
     {
         const int* src = reinterpret_cast<const int*>(runs + tr.x);
         int* dst = reinterpret_cast<int*>(&R);
         for (int k = threadIdx.x; k < int(sizeof(BandRun) / sizeof(int)); k += blockDim.x) dst[k] = src[k];
     }
     __syncthreads();
-    band_tile<LAT, S, false, MONO>(R.G, R.O, R.B, R.E, static_cast<const S*>(R.f[par_t]),
-                      static_cast<S*>(R.f[par_t ^ 1]), par_t, tr.y);
+    const S* fin = static_cast<const S*>(R.f[par_t]);
+    S* f = static_cast<S*>(R.f[par_t ^ 1]);
+    if constexpr (band_mono<S>()) band_tile_mono<LAT, S, false, false>(R.G, R.O, R.B, R.E, fin, f, par_t, tr.y);
+    else band_tile<LAT, S, false>(R.G, R.O, R.B, R.E, fin, f, par_t, tr.y);
 }
 
 // Zero gradient (Eq. zg-bc): the post-collision populations of x_f.
@@ -928,10 +1040,10 @@ int boundary_t(const Geom& G, const Offsets& O, const Export& E, const Band& B, 
     S* fo = static_cast<S*>(fnew);
     constexpr bool mono = band_mono<S>();
     constexpr int ncl = mono ? 1 : kCluster;
-    const dim3 grd(mono ? std::max(1, std::min(B.grid, B.n_tiles)) : B.n_tiles * ncl), blk(band_threads<mono>());
+    const dim3 grd(mono ? std::max(1, std::min(B.grid, B.n_tiles)) : B.n_tiles * ncl), blk(band_threads<S>());
     if (G.ref)
-        return launch_ex_cl(k_band<LAT, S, true, mono>, grd, blk, smem, st, false, ncl, G, O, B, E, fi, fo, par_t);
-    return launch_ex_cl(k_band<LAT, S, false, mono>, grd, blk, smem, st, false, ncl, G, O, B, E, fi, fo, par_t);
+        return launch_ex_cl(k_band<LAT, S, true>, grd, blk, smem, st, false, ncl, G, O, B, E, fi, fo, par_t);
+    return launch_ex_cl(k_band<LAT, S, false>, grd, blk, smem, st, false, ncl, G, O, B, E, fi, fo, par_t);
 }
 
 template <int LAT, typename S>
@@ -941,7 +1053,7 @@ int band_batch_t(const BandRun* runs, const int2* tile_run, int n_tiles, size_t 
     if (n_tiles == 0) return 0;
     constexpr bool mono = band_mono<S>();
     return launch_ex_cl(k_band_batch<LAT, S>, dim3(mono ? n_tiles : n_tiles * kCluster),
-                        dim3(band_threads<mono>()), smem, st, early, mono ? 1 : kCluster, runs, tile_run, par_t);
+                        dim3(kTileThreads), smem, st, early, mono ? 1 : kCluster, runs, tile_run, par_t);
 }
 
 template <int LAT, typename S>
@@ -959,8 +1071,7 @@ int prepare_t(const Band& B)
     auto set = [&](const void* k) {
         return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) == cudaSuccess;
     };
-    constexpr bool mono = band_mono<S>();
-    const bool ok = set((const void*)k_band<LAT, S, false, mono>) && set((const void*)k_band<LAT, S, true, mono>);
+    const bool ok = set((const void*)k_band<LAT, S, false>) && set((const void*)k_band<LAT, S, true>);
     return ok ? 0 : -1;
 }
 

@@ -431,9 +431,11 @@ __device__ void unknown_rhs(const Geom& G, const Band& B, const Relax<T>& P, con
 // the bulk neighbour after its collision, f*(x_f) - f^eq(U(x_f, t+1)), or
 // (dirichlet 2) that part projected onto the Hermite polynomials of orders 2
 // and 3 (a regularised scheme, named by the paper as future work).
-// Computed in the arithmetic type of the storage.
-template <int LAT, typename S, typename R, bool REF = true>
-__device__ void dirichlet(const Geom& G, const Band& B, S* f, const R* Us, const S* fsrc,
+// Computed in the arithmetic type of the storage.  PART of NPART: only every
+// NPART-th opposite pair from PART on (and the rest velocity for PART 0), so
+// that several threads can share one unknown's populations.
+template <int LAT, typename S, typename R, bool REF = true, int PART = 0, int NPART = 1>
+__device__ __forceinline__ void dirichlet(const Geom& G, const Band& B, S* f, const R* Us, const S* fsrc,
                           const UDesc& D, const R* Unew, bool dry = false)
 {
     // dry: the same instructions without the stores (instruction-cache
@@ -442,6 +444,7 @@ __device__ void dirichlet(const Geom& G, const Band& B, S* f, const R* Us, const
     // populations, indexed by velocity (both read only for Eq. NEEP)
     using L = Lat<LAT>;
     using Cm = typename Store<S>::C;
+    auto mine = [](int i) { return (i == 0 ? 0 : (i - 1) / 2 % NPART) == PART; };
     Moments<LAT, Cm> m;
     m.s0 = Cm(Unew[0]);
     m.rho = Cm(G.rho0) + m.s0;
@@ -473,14 +476,19 @@ __device__ void dirichlet(const Geom& G, const Band& B, S* f, const R* Us, const
         }
         Cm gs[L::Q];
         equilibrium<LAT, Cm>(ms, gs);
-        Cm gn[L::Q];
-#pragma unroll
-        for (int i = 0; i < L::Q; ++i) {
+        auto neq = [&](int i) -> Cm {
             Cm v = Cm(Store<S>::value(fsrc[i]));     // fsrc is in shared memory
             if (Store<S>::SCALED) v *= Cm(L::w(i));
-            gn[i] = v - gs[i];
-        }
-        if (B.dirichlet == 2) {
+            return v - gs[i];
+        };
+        if (B.dirichlet != 2) {
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i)
+                if (mine(i)) ge[i] += neq(i);
+        } else {
+            Cm gn[L::Q];
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i) gn[i] = neq(i);
             // Regularised form: the Hermite projection of f^neq onto orders 2
             // (and 3 on the thermal lattices),
             // w_i [H2_i : a2 / (2 c_s^4) + H3_i : a3 / (6 c_s^6)], a_n = sum H_n f^neq
@@ -511,11 +519,9 @@ __device__ void dirichlet(const Geom& G, const Band& B, S* f, const R* Us, const
                                   (cy * cy * cy - Cm(3) * cs2 * cy) * a3yyy;
                     h += h3 / (Cm(6) * cs2 * cs2 * cs2);
                 }
-                gn[i] = Cm(L::w(i)) * h;
+                if (mine(i)) ge[i] += Cm(L::w(i)) * h;
             }
         }
-#pragma unroll
-        for (int i = 0; i < L::Q; ++i) ge[i] += gn[i];
     }
     const int nb = D.kind >= 4 ? G.M : 1;
     for (int a = 0; a < nb; ++a)
@@ -523,6 +529,7 @@ __device__ void dirichlet(const Geom& G, const Band& B, S* f, const R* Us, const
             const long long node = D.wnode + a * D.wdx + b * D.wdy;
 #pragma unroll
             for (int i = 0; i < L::Q; ++i) {
+                if (!mine(i)) continue;
                 Cm v = ge[i];
                 if (Store<S>::SCALED) v *= Cm(1.0 / L::w(i));
                 if (!dry) Store<S>::put(f + L::plane_of(i) * G.plane + node, v);
