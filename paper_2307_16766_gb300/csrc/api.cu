@@ -778,21 +778,22 @@ int mark(lbm_handle* h, int k, cudaStream_t st)
 }
 
 // Bulk update of step (parity par) on stream st, bracketed by the caller's
-// timing events 0 and 1 when set; early: start beside the band kernel just
-// launched on st (programmatic stream serialization).
-int bulk(lbm_handle* h, int par, cudaStream_t st, bool early = false)
+// timing events 0 and 1 when set; chain: how it follows the kernel before it
+// on st (launch_bulk).
+int bulk(lbm_handle* h, int par, cudaStream_t st, int chain = CHAIN_NONE)
 {
     int rc = mark(h, 0, st);
     if (rc != LBM_OK) return rc;
     rc = launch_bulk(h->lattice, h->storage, h->G, h->O, h->bulk, h->tmap[par], h->f[par],
-                     h->f[par ^ 1], h->flag + 1, st, early);
+                     h->f[par ^ 1], h->flag + 1, st, chain);
     if (rc) return check_launch(h, rc, "bulk kernel");
     return mark(h, 1, st);
 }
 
 // Inflow equilibrium (once per buffer) and the band kernel of step (parity
-// par) on stream st, bracketed by timing events 3 and 4.
-int band(lbm_handle* h, int par, cudaStream_t st)
+// par) on stream st, bracketed by timing events 3 and 4; early: the band
+// kernel may start beside the previous step's bulk update.
+int band(lbm_handle* h, int par, cudaStream_t st, bool early = false)
 {
     int rc = mark(h, 3, st);
     if (rc != LBM_OK) return rc;
@@ -802,11 +803,12 @@ int band(lbm_handle* h, int par, cudaStream_t st)
     if (h->n_inflow > 0 && !h->inflow_done[par ^ 1]) {
         rc = launch_inflow(h->lattice, h->storage, h->G, h->inflow_nodes, h->n_inflow, h->Uin,
                            h->f[par ^ 1], st);
+        early = false;                  // the band kernel comes after that one
         if (rc) return check_launch(h, rc, "inflow kernel");
         h->inflow_done[par ^ 1] = true;
     }
     rc = launch_boundary(h->lattice, h->storage, h->G, h->O, h->E, h->B, h->f[par], h->f[par ^ 1],
-                         par, st);
+                         par, st, early);
     if (rc) return check_launch(h, rc, "band kernel");
     return mark(h, 4, st);
 }
@@ -1026,13 +1028,21 @@ int lbm_step(lbm_handle* h, int n)
     }
     if (h->bulk_pending) { h->err = "lbm_step in the middle of a phased step"; return LBM_ERR_STATE; }
     if (h->grad_stale) { h->err = kGradStale; return LBM_ERR_STATE; }
+    // From the second step on, a step's first kernel is launched early: its
+    // launch and its reads of fixed data run beside the previous step's bulk
+    // update, whose completion it waits for.
+    bool timed = false;
+    for (int k = 0; k < 5; ++k) timed = timed || h->kev[k];
     for (int i = 0; i < n; ++i) {
         const int par = int(h->steps & 1);
         int rc = mark(h, 2, h->stream);
         if (rc != LBM_OK) return rc;
+        bool early = i > 0 && !timed && h->B.n_zg == 0;
         if (h->B.n_tiles == 0) {
             // no characteristic side: bulk, inflow and zero gradient in order
-            rc = bulk(h, par, h->stream);
+            // (no early start after an inflow kernel)
+            if (h->n_inflow > 0 && !(h->inflow_done[0] && h->inflow_done[1])) early = false;
+            rc = bulk(h, par, h->stream, early ? CHAIN_BULK : CHAIN_NONE);
             if (rc == LBM_OK) rc = band(h, par, h->stream);
             if (rc == LBM_OK) rc = zero_gradient(h, par, h->stream);
             if (rc != LBM_OK) return rc;
@@ -1046,8 +1056,8 @@ int lbm_step(lbm_handle* h, int n)
         // kernel allows at once; the zero-gradient copies and the next step
         // wait for both.
         if (!h->kev[0] && !h->kev[3]) {
-            rc = band(h, par, h->stream);
-            if (rc == LBM_OK) rc = bulk(h, par, h->stream, true);
+            rc = band(h, par, h->stream, early);
+            if (rc == LBM_OK) rc = bulk(h, par, h->stream, CHAIN_BAND);
             if (rc == LBM_OK) rc = zero_gradient(h, par, h->stream);
             if (rc != LBM_OK) return rc;
             h->steps++;

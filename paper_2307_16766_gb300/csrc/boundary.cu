@@ -246,7 +246,7 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
     constexpr bool TH = L::THERMAL;
     // a kernel launched after this one for early start (the bulk update,
     // which reads only the old buffer) may begin now
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_trigger();
     constexpr int kPull = WIDE ? 2 * kTileThreads : kTileThreads;      // threads of the strip phase
     const int tid = int(threadIdx.x), l = tid % kTileThreads, warp = tid / 32;
     const bool dry = WIDE && warp >= kPull / 32;
@@ -553,7 +553,7 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
 //    mask of time t.
 // 3. The owners write U(t + 1) and the mesoscopic Dirichlet populations
 //    (equilibrium or Eq. NEEP), shared out over the four groups.
-template <int LAT, typename S, bool REF>
+template <int LAT, typename S, bool REF, bool BATCH>
 __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const Band& B,
                                           const Export& E, const S* __restrict__ fin,
                                           S* __restrict__ f, int par_t, int tile)
@@ -562,9 +562,7 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     using C = typename Store<S>::C;
     using R = typename StripReal<S>::T;
     constexpr bool TH = L::THERMAL;
-    // a kernel launched after this one for early start (the bulk update,
-    // which reads only the old buffer) may begin now
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (BATCH) pdl_trigger();           // as band_tile_mono (a batch's kernels start with the old step complete)
     static_assert(sizeof(R) == 8, "FP32 / FP16 storage takes band_tile_mono");
     const int grp = int(cg::this_cluster().block_rank());
     const int l = int(threadIdx.x);
@@ -628,6 +626,13 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     const int nc0 = __syncthreads_count(D.level <= 3), nc1 = __syncthreads_count(D.level <= 2),
               nc2 = __syncthreads_count(D.level <= 1), nc3 = __syncthreads_count(D.level <= 0);
     sync_all();                         // every CTA of the cluster runs before any remote store
+    if (!BATCH) {
+        // Fixed data so far: this kernel starts beside the previous step's
+        // bulk update.  Once that step is complete, the bulk update of this
+        // one (which reads only the old buffer) may begin.
+        pdl_wait();
+        pdl_trigger();
+    }
 
     // 1. strip nodes: macros of t and moments of t for every CTA; macros of
     //    t + 1 (pull and Eq. macro) by CTA k % kCluster for node k, shared out;
@@ -984,7 +989,7 @@ __global__ void __launch_bounds__(band_threads<S>(), 1)
             __syncthreads();            // the next tile reuses the shared memory
         }
     } else {
-        band_tile<LAT, S, REF>(G, O, B, E, fin, f, par_t, blockIdx.x / kCluster);
+        band_tile<LAT, S, REF, false>(G, O, B, E, fin, f, par_t, blockIdx.x / kCluster);
     }
 }
 
@@ -1009,7 +1014,7 @@ __global__ void __launch_bounds__(kTileThreads, band_mono<S>() ? 4 : 1)
     const S* fin = static_cast<const S*>(R.f[par_t]);
     S* f = static_cast<S*>(R.f[par_t ^ 1]);
     if constexpr (band_mono<S>()) band_tile_mono<LAT, S, false, false>(R.G, R.O, R.B, R.E, fin, f, par_t, tr.y);
-    else band_tile<LAT, S, false>(R.G, R.O, R.B, R.E, fin, f, par_t, tr.y);
+    else band_tile<LAT, S, false, true>(R.G, R.O, R.B, R.E, fin, f, par_t, tr.y);
 }
 
 // Zero gradient (Eq. zg-bc): the post-collision populations of x_f.
@@ -1032,18 +1037,24 @@ size_t band_smem(const Band& B)
 
 template <int LAT, typename S>
 int boundary_t(const Geom& G, const Offsets& O, const Export& E, const Band& B, const void* fin,
-               void* fnew, int par_t, cudaStream_t st)
+               void* fnew, int par_t, cudaStream_t st, bool early)
 {
     if (B.n_tiles == 0) return 0;
     const size_t smem = band_smem<LAT, S>(B);
     const S* fi = static_cast<const S*>(fin);
     S* fo = static_cast<S*>(fnew);
     constexpr bool mono = band_mono<S>();
+    // Early start for the FP64 form only (D2Q9 64^2: 31.2 us a step without,
+    // 28.3 us with; D2Q17 200x20: 44.2, 42.0).  The chain of completions it
+    // waits for (band, bulk, then this kernel) takes longer than a launch
+    // when the band kernel is short: FP32 256^2 20.6 us a step without,
+    // 22.2 us with; 1024x512 34.2, 38.9.
+    early = early && !mono;
     constexpr int ncl = mono ? 1 : kCluster;
     const dim3 grd(mono ? std::max(1, std::min(B.grid, B.n_tiles)) : B.n_tiles * ncl), blk(band_threads<S>());
     if (G.ref)
-        return launch_ex_cl(k_band<LAT, S, true>, grd, blk, smem, st, false, ncl, G, O, B, E, fi, fo, par_t);
-    return launch_ex_cl(k_band<LAT, S, false>, grd, blk, smem, st, false, ncl, G, O, B, E, fi, fo, par_t);
+        return launch_ex_cl(k_band<LAT, S, true>, grd, blk, smem, st, early, ncl, G, O, B, E, fi, fo, par_t);
+    return launch_ex_cl(k_band<LAT, S, false>, grd, blk, smem, st, early, ncl, G, O, B, E, fi, fo, par_t);
 }
 
 template <int LAT, typename S>
@@ -1103,9 +1114,9 @@ int zg_t(const Geom& G, const Band& B, void* fnew, cudaStream_t st)
     } while (0)
 
 int launch_boundary(int lat, int storage, const Geom& G, const Offsets& O, const Export& E,
-                    const Band& B, const void* fin, void* fnew, int par_t, cudaStream_t st)
+                    const Band& B, const void* fin, void* fnew, int par_t, cudaStream_t st, bool early)
 {
-#define CALL(L, S) boundary_t<L, S>(G, O, E, B, fin, fnew, par_t, st)
+#define CALL(L, S) boundary_t<L, S>(G, O, E, B, fin, fnew, par_t, st, early)
     BAND_DISPATCH(lat, storage, CALL);
 #undef CALL
     return -1;

@@ -162,7 +162,7 @@ constexpr int bulk_rows() { return (sizeof(S) <= 4 && !REF) ? 2 : 1; }
 
 template <int LAT, typename S, bool REF>
 __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const Offsets& O, const Region& R,
-                                          const S* __restrict__ fin, S* __restrict__ fout, int* status)
+                                          const S* __restrict__ fin, S* __restrict__ fout, int* status, int chain)
 {
     constexpr int ROWS = bulk_rows<S, REF>();
     using L = Lat<LAT>;
@@ -189,6 +189,7 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[r])));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (chain == CHAIN_BULK) pdl_wait();
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             if (!staged(yb + r)) continue;
@@ -199,6 +200,7 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
                                  std::make_integer_sequence<int, L::NG>{});
         }
     }
+    if (chain == CHAIN_BULK) pdl_wait();
     __syncthreads();
 #pragma unroll 1
     for (int r = 0; r < ROWS; ++r) {
@@ -224,12 +226,25 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
     }
 }
 
+// The next step's first kernel may be launched once every CTA of this grid
+// has begun (it waits for this grid's completion): periodic D2Q37 2048x1024
+// FP32 106.6 us a step without, 104.5 us with.  Beside a band kernel
+// (CHAIN_BAND) the last CTA stays until that kernel is complete, so that this
+// grid's completion stands for the whole step's.
+__device__ __forceinline__ void bulk_end(int chain)
+{
+    if (chain == CHAIN_BAND && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && threadIdx.x == 0)
+        pdl_wait();
+}
+
 template <int LAT, typename S>
 __global__ void __launch_bounds__(kBulkThreads)
     k_bulk(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
-           S* __restrict__ fout, int* status)
+           S* __restrict__ fout, int* status, int chain)
 {
-    bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status);
+    pdl_trigger();
+    bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status, chain);
+    bulk_end(chain);
 }
 
 // With a reference equilibrium: about twice the equilibrium arithmetic per
@@ -238,9 +253,11 @@ __global__ void __launch_bounds__(kBulkThreads)
 template <int LAT, typename S>
 __global__ void __launch_bounds__(kBulkThreads)
     k_bulk_ref(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
-               S* __restrict__ fout, int* status)
+               S* __restrict__ fout, int* status, int chain)
 {
-    bulk_body<LAT, S, true>(tm, G, O, R, fin, fout, status);
+    pdl_trigger();
+    bulk_body<LAT, S, true>(tm, G, O, R, fin, fout, status, chain);
+    bulk_end(chain);
 }
 
 // Persistent form of k_bulk for one or many grids of one lattice and
@@ -547,7 +564,7 @@ int inflow_t(const Geom& G, const int* nodes, int n, const double U[4], void* f,
 
 template <int LAT, typename S>
 int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* tmaps,
-           const void* fin, void* fout, int* status, cudaStream_t st, bool early)
+           const void* fin, void* fout, int* status, cudaStream_t st, int chain)
 {
     const int h = R.y1 - R.y0;
     if (R.x1 <= R.x0 || h <= 0) return 0;
@@ -559,18 +576,19 @@ int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* 
     tm.m2 = tmaps[3];
     tm.m1 = tmaps[4];
     const dim3 blk(kBulkThreads);
+    const bool early = chain != CHAIN_NONE;
     if (G.ref) {
         constexpr int ROWS = bulk_rows<S, true>();
         constexpr size_t smem = ROWS * Stage<LAT, S>::TOTAL;
         static_assert(smem <= 48 * 1024, "bulk staging above the default dynamic shared memory");
         return launch_ex(k_bulk_ref<LAT, S>, dim3(t1 - t0, (h + ROWS - 1) / ROWS), blk, smem, st, early, tm, G, O,
-                         R, static_cast<const S*>(fin), static_cast<S*>(fout), status);
+                         R, static_cast<const S*>(fin), static_cast<S*>(fout), status, chain);
     }
     constexpr int ROWS = bulk_rows<S, false>();
     constexpr size_t smem = ROWS * Stage<LAT, S>::TOTAL;
     static_assert(smem <= 48 * 1024, "bulk staging above the default dynamic shared memory");
     return launch_ex(k_bulk<LAT, S>, dim3(t1 - t0, (h + ROWS - 1) / ROWS), blk, smem, st, early, tm, G, O, R,
-                     static_cast<const S*>(fin), static_cast<S*>(fout), status);
+                     static_cast<const S*>(fin), static_cast<S*>(fout), status, chain);
 }
 
 template <int LAT, typename S>
@@ -638,9 +656,9 @@ int launch_inflow(int lat, int storage, const Geom& G, const int* nodes, int n, 
 
 int launch_bulk(int lat, int storage, const Geom& G, const Offsets& O, const Region& R,
                 const CUtensorMap* tmaps, const void* fin, void* fout, int* status,
-                cudaStream_t st, bool early)
+                cudaStream_t st, int chain)
 {
-#define CALL(L, S) bulk_t<L, S>(G, O, R, tmaps, fin, fout, status, st, early)
+#define CALL(L, S) bulk_t<L, S>(G, O, R, tmaps, fin, fout, status, st, chain)
     LBM_DISPATCH(lat, storage, CALL);
 #undef CALL
 }

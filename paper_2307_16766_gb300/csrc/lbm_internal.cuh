@@ -610,6 +610,16 @@ struct Export {
     void* stripN;
 };
 
+// Programmatic launches of one step after the other (lbm_step).  A kernel
+// launched early (launch_ex) may begin once every CTA of the kernel before it
+// has called pdl_trigger() or left; pdl_wait() returns when that kernel has
+// completed and its writes are visible (at once if not launched early).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// How a bulk launch follows the kernel before it in the stream (see lbm_step).
+enum { CHAIN_NONE = 0, CHAIN_BAND = 1, CHAIN_BULK = 2 };
+
 // Shared-memory address of a generic pointer, and the global nanosecond
 // timer (for bounded waits).
 __device__ __forceinline__ unsigned smem_u32(const void* p)
@@ -797,19 +807,21 @@ int launch_inflow(int lat, int storage, const Geom& G, const int* nodes, int n, 
                   void* f, cudaStream_t st);
 // One bulk step fin -> fout over the nodes of region R; tmaps[0..4] describe
 // fin for the tensor copies (box depths 7, 5, 3, 2, 1 planes); *status gets bit 1
-// if a copy never completed.  early: programmatic stream serialization (the
-// launch may start while the kernel before it in the stream runs, once that
-// kernel's CTAs have signalled; it must not read what that kernel writes).
+// if a copy never completed.  chain: CHAIN_NONE (ordinary launch),
+// CHAIN_BAND (starts early beside the band kernel of the same step, whose
+// CTAs signal after the previous step is complete) or CHAIN_BULK (starts early
+// after the previous step's bulk kernel and waits for it).
 int launch_bulk(int lat, int storage, const Geom& G, const Offsets& O, const Region& R,
                 const CUtensorMap* tmaps, const void* fin, void* fout, int* status,
-                cudaStream_t st, bool early = false);
+                cudaStream_t st, int chain = CHAIN_NONE);
 int launch_macros(int lat, int storage, const Geom& G, const void* f, double* rho, double* ux,
                   double* uy, double* T, int* flag, cudaStream_t st);
 // The band of one step fin -> fnew: strip nodes, RK4 of the characteristic
-// boundary state, Dirichlet populations.
+// boundary state, Dirichlet populations.  early: the launch may start beside
+// the previous step's bulk kernel (CHAIN_BAND), whose completion it waits for.
 int launch_boundary(int lat, int storage, const Geom& G, const Offsets& O, const Export& E,
                     const Band& B, const void* fin, void* fnew, int par_t,
-                    cudaStream_t st);
+                    cudaStream_t st, bool early = false);
 // One grid of the batched band kernel, in device memory.
 struct BandRun {
     Geom G;
