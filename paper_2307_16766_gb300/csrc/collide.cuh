@@ -50,24 +50,66 @@ __device__ __forceinline__ Moments<LAT, C> moments_G(const Geom& G, const C* g)
 // Viscous stress sigma' = -(1 - 1/(2 tau)) sum c c (f - f^eq) (Eq. LaplaceU)
 // and heat flux q = (1 - 1/(2 tau)) 1/2 sum (f - f^eq) |c-u|^2 (c-u)
 // (Eqs. heatflux, LaplaceT; the equilibrium part of the central third
-// moment vanishes on the thermal lattices).  The equilibria reproduce the
-// Maxwellian moments through third order (second on D2Q9), so their share is
-// taken in closed form,
+// moment vanishes on the thermal lattices).
+// FP64: the equilibria reproduce the Maxwellian moments through third order
+// (second on D2Q9), so their share is taken in closed form,
 //   sum f^eq c_a c_b = rho (u_a u_b + c_s^2 theta delta_ab),
 //   sum f^eq |c|^2 c_a = rho u_a (|u|^2 + 4 c_s^2 theta),
-// instead of from 37 evaluated populations (which took 500 more operations a
-// node, 30 us of FP64 issue in a band tile).  f - f^eq carries no mass,
-// momentum or energy: on the thermal lattices its stress is traceless, formed
-// from c_x^2 - c_y^2 with the large isotropic part cancelling pair by pair,
-// and its third moment is that of (|c|^2 - 4 c_s^2) c, so that the rounding
-// of rho, u and theta does not enter at their size (a boundary at rest
-// amplifies such noise).  With a reference the closed forms are differences
-// from the reference's.
+// instead of from 37 evaluated populations (500 more operations a node, 30 us
+// of FP64 issue in a band tile).  f - f^eq carries no mass, momentum or
+// energy: on the thermal lattices its stress is traceless, formed from
+// c_x^2 - c_y^2 with the large isotropic part cancelling pair by pair, and its
+// third moment is that of (|c|^2 - 4 c_s^2) c, so that the rounding of rho, u
+// and theta does not enter at their size.  With a reference the closed forms
+// are differences from the reference's.
+// FP32 keeps the sums over g - g^eq: the closed form is faster where the band
+// kernel is all there is (256^2: 2.12 ms a pass, 2.20 with the sums) and
+// slower beside a large bulk (1024x512: 3.48, 3.34; 96 runs: 30.5, 29.8), and
+// the gradients of short runs feel its different rounding.
+// FP32 and derivative numbers: from the evaluated equilibrium.
+template <int LAT, typename C, typename T>
+__device__ __forceinline__ void neq_evaluated(const C* g, const Moments<LAT, C>& m, T fac, T* N)
+{
+    using L = Lat<LAT>;
+    Moments<LAT, C> me = m;
+    if constexpr (std::is_same_v<C, float>)
+        // kept apart from the moments' and the collision's arithmetic, so that
+        // every kernel contracts this one alike (a run of a batch repeats bit
+        // for bit alone)
+        asm volatile("" : "+f"(me.s0), "+f"(me.rho), "+f"(me.ux), "+f"(me.uy), "+f"(me.dT));
+    C geq[L::Q];
+    equilibrium<LAT, C>(me, geq);
+    C pxx = 0, pxy = 0, pyy = 0, qx = 0, qy = 0;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const C d = g[i] - geq[i];
+        const C cx = C(L::cx(i)), cy = C(L::cy(i));
+        pxx += cx * cx * d;
+        pxy += cx * cy * d;
+        pyy += cy * cy * d;
+        if (L::THERMAL) {
+            const C ex = cx - me.ux, ey = cy - me.uy;
+            const C h = C(0.5) * d * (ex * ex + ey * ey);
+            qx += h * ex;
+            qy += h * ey;
+        }
+    }
+    N[0] = -fac * T(pxx);
+    N[1] = -fac * T(pxy);
+    N[2] = -fac * T(pyy);
+    N[3] = fac * T(qx);
+    N[4] = fac * T(qy);
+}
+
+template <int LAT, typename C, typename T>
+__device__ __forceinline__ void neq_close(const Moments<LAT, C>& m, T fac, T* N, C pxy, C dxy, C pxx, C pyy, C rx, C ry);
+
 template <int LAT, typename C, typename T>
 __device__ __forceinline__ void neq_moments(const C* g, const Moments<LAT, C>& m, T fac, T* N)
 {
     using L = Lat<LAT>;
     constexpr double cs2 = L::CS2;
+    if constexpr (!std::is_same_v<C, double>) return neq_evaluated<LAT, C, T>(g, m, fac, N);
     // sum g c_x c_y; sum g (c_x^2 - c_y^2) per class (thermal) or sum g c_a^2
     // (D2Q9); sum g (|c|^2 - 4 c_s^2) c_a
     C pxy = 0, dxy = 0, pxx = 0, pyy = 0, rx = 0, ry = 0;
@@ -95,6 +137,15 @@ __device__ __forceinline__ void neq_moments(const C* g, const Moments<LAT, C>& m
         const int c2 = L::c2cls(k), dd = c2 == 1 ? 1 : c2 == 4 ? 4 : c2 == 5 ? 3 : c2 == 9 ? 9 : c2 == 10 ? 8 : 0;
         if (L::THERMAL && dd) dxy += C(dd) * d;
     }
+    neq_close<LAT, C, T>(m, fac, N, pxy, dxy, pxx, pyy, rx, ry);
+}
+
+// The closed-form equilibrium's share taken from the sums above.
+template <int LAT, typename C, typename T>
+__device__ __forceinline__ void neq_close(const Moments<LAT, C>& m, T fac, T* N, C pxy, C dxy, C pxx, C pyy, C rx, C ry)
+{
+    using L = Lat<LAT>;
+    constexpr double cs2 = L::CS2;
     const C ux = m.ux, uy = m.uy;
     if (m.ref) {
         const C U2x = m.Ux * m.Ux, U2y = m.Uy * m.Uy, wx = m.vx * (ux + m.Ux), wy = m.vy * (uy + m.Uy);
