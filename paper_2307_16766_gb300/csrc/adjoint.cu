@@ -60,19 +60,12 @@ template <typename S>
 using RT = typename StripReal<S>::T;      // boundary solver inputs
 
 constexpr int kAdjThreads = 128;
-// The cooperative boundary kernel: two CTAs of six warps per SM (at most 170
-// registers a thread), so that one stage's derivative items (eight per
-// unknown) and the next step's stage items run in one pass of the grid.
+// The cooperative boundary kernel: one CTA of six warps per SM (one item per
+// unknown and phase: a few thousand), with at most 170 registers a thread, so
+// that it leaves half of the SM to the bulk kernel on the other stream.
 constexpr int kBandThreads = 192;
-// Forward derivative directions per evaluation: four, so that one boundary
-// unknown's right-hand side is differentiated by eight threads within the
-// register cap of kBandThreads (eight directions per thread spilled and ran
-// 4x slower; two needed two passes of the grid per stage).
+// Forward derivative directions per evaluation of the "-FD" viscous vector.
 constexpr int kChunk = 4;
-constexpr int kRhsInputs = 29;            // 5 stage-field neighbours x 4, V (4), theta (5)
-constexpr int kRhsChunks = (kRhsInputs + kChunk - 1) / kChunk;
-constexpr int kMesoInputs = 36;           // 5 stencil nodes x (5 moments, u_x, u_y), drho of node 0
-constexpr int kMesoChunks = (kMesoInputs + kChunk - 1) / kChunk;
 constexpr int kFdInputs = 24;             // 6 neighbours x 4
 constexpr int kFdChunks = kFdInputs / kChunk;
 
@@ -87,52 +80,71 @@ __device__ __forceinline__ bool wrap_bulk(const Geom& G, int& x, int& y)
 
 // a[k] = sum_i lam(i) d g^eq_i / d m_k at the moments m = (drho, u_x, u_y,
 // theta - 1): the equilibrium (Eqs. feq-3, feq-4, pairwise as equilibrium()
-// evaluates it) on forward derivatives along the four moments.
+// evaluates it) backwards.  Per pair, with lambda_(+-) = lam(i) +- lam(i + 1),
+//   ev = a0 + p^2 (a2 + a4 p^2),  od = p (a1 + a3 p^2),
+//   sum lam g = w (lambda_+ (s0 + rho ev) + lambda_- rho od),
+// about 20 operations, against 65 on forward derivatives along the four
+// moments (k_adj_bulk<D2Q37, FP32> 512x256: 33.9 us, now 22.7 us).
 template <int LAT, typename C, typename Lam>
 __device__ __forceinline__ void eq_vjp(C s0, C ux, C uy, C dT, C rho0, Lam&& lam, C a[4])
 {
     using L = Lat<LAT>;
-    using D4 = Dual<C, 4>;
-    D4 m0(s0), mx(ux), my(uy), mt(L::THERMAL ? dT : C(0));
-    m0.d[0] = C(1);
-    mx.d[1] = C(1);
-    my.d[2] = C(1);
-    if (L::THERMAL) mt.d[3] = C(1);
-    const D4 rho = D4(rho0) + m0;
+    const C t = L::THERMAL ? dT : C(0), rho = rho0 + s0;
     constexpr C ics2 = C(1.0 / L::CS2);
     constexpr C a3 = L::ORDER >= 3 ? C(1.0 / 6.0) : C(0);
     constexpr C a4 = L::ORDER >= 4 ? C(1.0 / 24.0) : C(0);
-    const D4 uxs = mx * ics2, uys = my * ics2;
-    const EqPoly<D4> e = eq_poly<LAT, D4>(mx * uxs + my * uys, mt);
-    C acc[4] = {C(0), C(0), C(0), C(0)};
-    auto add = [&](C l, const D4& g) {
+    const C uxs = ux * ics2, uys = uy * ics2, u2 = ux * uxs + uy * uys;
+    const EqPoly<C> e = eq_poly<LAT, C>(u2, t);
+    // adjoints (over rho) of the coefficients and of uxs, uys; bs, br of s0, rho
+    const C l0 = C(L::w(0)) * lam(0);
+    C A0 = l0, B0 = 0, C0 = 0, A1 = 0, B1 = 0, A2 = 0, B2 = 0, X = 0, Y = 0, bs = l0, br = l0 * e.A0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] += l * g.d[k];
-    };
-    {
-        const D4 g0 = C(L::w(0)) * (m0 + rho * e.A0);
-        add(lam(0), g0);
-    }
-#pragma unroll
-    for (int i = 1; i < L::Q; i += 2) {
-        const int k = L::cls(i);
+    for (int k = 1; k < L::NCLS; ++k) {
         const C xi2 = C(L::c2cls(k)) * ics2;
-        const D4 A0 = e.A0 + xi2 * (e.B0 + e.C0 * xi2);
-        const D4 A1 = e.A1 + e.B1 * xi2;
-        const D4 A2 = e.A2 + e.B2 * xi2;
-        D4 p;
-        if (L::cx(i) == 0) p = C(L::cy(i)) * uys;
-        else if (L::cy(i) == 0) p = C(L::cx(i)) * uxs;
-        else p = C(L::cx(i)) * uxs + C(L::cy(i)) * uys;
-        const D4 p2 = p * p;
-        const D4 ev = A0 + p2 * (A2 + p2 * a4);
-        const D4 od = p * (A1 + p2 * a3);
-        const D4 ws0 = C(L::w(i)) * m0, wr = C(L::w(i)) * rho;
-        add(lam(i), ws0 + wr * (ev + od));
-        add(lam(i + 1), ws0 + wr * (ev - od));
-    }
+        const C c0 = e.A0 + xi2 * (e.B0 + e.C0 * xi2), c1 = e.A1 + e.B1 * xi2, c2 = e.A2 + e.B2 * xi2;
+        C s0k = 0, s1k = 0, s2k = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] = acc[k];
+        for (int i = 1; i < L::Q; i += 2) {
+            if (L::cls(i) != k) continue;
+            const C lp = lam(i), lm = lam(i + 1), le = C(L::wcls(k)) * (lp + lm), lo = C(L::wcls(k)) * (lp - lm);
+            C p;
+            if (L::cx(i) == 0) p = C(L::cy(i)) * uys;
+            else if (L::cy(i) == 0) p = C(L::cx(i)) * uxs;
+            else p = C(L::cx(i)) * uxs + C(L::cy(i)) * uys;
+            const C p2 = p * p, f = c1 + p2 * a3, lop = lo * p;
+            bs += le;
+            br += le * (c0 + p2 * (c2 + p2 * a4)) + lop * f;
+            s0k += le;
+            s1k += lop;
+            s2k += le * p2;
+            // d/dp
+            const C d = C(2) * p * (le * (c2 + C(2) * a4 * p2) + a3 * lop) + lo * f;
+            if (L::cx(i)) X += C(L::cx(i)) * d;
+            if (L::cy(i)) Y += C(L::cy(i)) * d;
+        }
+        A0 += s0k;
+        B0 += xi2 * s0k;
+        C0 += (xi2 * xi2) * s0k;
+        A1 += s1k;
+        B1 += xi2 * s1k;
+        A2 += s2k;
+        B2 += xi2 * s2k;
+    }
+    // eq_poly backwards
+    C bu = C(-0.5) * A0, bt = C(0);
+    if (L::ORDER == 3) {
+        bu -= C(0.5) * A1;
+        bt = C(0.5) * (B0 + B1) - A0 - C(2) * A1;
+    } else if (L::THERMAL) {
+        bu += A0 * (C(0.25) * u2 + t) - C(0.25) * (t * B0 + A2) - C(0.5) * A1;
+        bt = A0 * (u2 + C(2) * t - C(1)) + B0 * (C(0.5) - C(0.25) * u2 - C(2) * t) + C(0.25) * (t * C0 + B2) +
+             C(0.5) * B1 - C(2) * A1 - C(1.5) * A2;
+    }
+    const C r = rho * ics2;
+    a[0] = bs + br;
+    a[1] = r * (C(2) * ux * bu + X);
+    a[2] = r * (C(2) * uy * bu + Y);
+    a[3] = L::THERMAL ? rho * bt : C(0);
 }
 
 // Pull-back of a covector mu on the moments m = (drho, u_x, u_y, theta - 1)
@@ -265,16 +277,15 @@ __global__ void __launch_bounds__(kAdjThreads)
 
 // lambda_U(t+1)[u] += sum over the nodes b the unknown writes and the
 // velocities i of lambda*_{t+1}(b, i) d f^eq_i / dU at U_b(t+1): per node,
-// sum_i lambda*_i dg^eq_i/dU_k of one node the Dirichlet write of unknown u
-// set (node q of a corner's M x M block, row-major; the node itself for a
-// side unknown), lambda*_i = lambda^pre_{t+2}(node + c_i, i), U = U_b(t+1).
+// out[k] = sum_i lambda*_i dg^eq_i/dU_k of one node the Dirichlet write of
+// unknown u set (node q of a corner's M x M block, row-major; the node itself
+// for a side unknown), lambda*_i = lambda^pre_{t+2}(node + c_i, i), U = U_b(t+1).
 template <int LAT, typename S>
-__device__ __forceinline__ CT<S> dirichlet_part(const Geom& G, const UDesc& D, const double* __restrict__ U,
-                                                const CT<S>* __restrict__ lnext, int k, int q)
+__device__ __forceinline__ void dirichlet_part(const Geom& G, const UDesc& D, const double* __restrict__ U,
+                                               const CT<S>* __restrict__ lnext, int q, CT<S>* out)
 {
     using L = Lat<LAT>;
     using C = CT<S>;
-    using D1 = Dual<C, 1>;
     const int a = q / G.M, b = q % G.M;
     const long long node = D.wnode + (D.kind >= 4 ? a * D.wdx + b * D.wdy : 0);
     const int x = int(node % G.nxp), y = int(node / G.nxp);
@@ -284,58 +295,43 @@ __device__ __forceinline__ CT<S> dirichlet_part(const Geom& G, const UDesc& D, c
         int xs = x + L::cx(i), ys = y + L::cy(i);
         lam[i] = wrap_bulk(G, xs, ys) ? lnext[L::plane_of(i) * G.plane + (long long)ys * G.nxp + xs] : C(0);
     }
-    Moments<LAT, D1> m;
-    m.s0 = D1(U[0]);
-    m.ux = D1(U[1]);
-    m.uy = D1(U[2]);
-    m.dT = D1(L::THERMAL ? U[3] : 0.0);
-    (k == 0 ? m.s0 : k == 1 ? m.ux : k == 2 ? m.uy : m.dT).d[0] = C(1);
-    m.rho = D1(G.rho0) + m.s0;
-    D1 ge[L::Q];
-    equilibrium<LAT, D1>(m, ge);
-    C s = C(0);
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) s += lam[i] * ge[i].d[0];
-    return s;
+    eq_vjp<LAT, C>(C(U[0]), C(U[1]), C(U[2]), C(U[3]), C(G.rho0), [&](int i) { return lam[i]; }, out);
 }
 
-// The Dirichlet write's adjoint, thread (u, k): lambda_U(t+1)_k of unknown
-// u gains the share of the node it writes (of the first node of a corner's
-// block; the other M^2 - 1 nodes of the four corner blocks are items of
-// adj_corner_item, folded in by the next phase in a fixed order), by
-// forward derivatives of the equilibrium along moment k; thread (u, 0)
-// also sets the stage-0 field Y0[u] = U_b(t).
+// The Dirichlet write's adjoint, item u: lambda_U(t+1) of unknown u gains
+// the share of the node it writes (of the first node of a corner's block; the
+// other M^2 - 1 nodes of the four corner blocks are items of
+// adj_corner_item, folded in by the next phase in a fixed order); also sets
+// the stage-0 field Y0[u] = U_b(t).
 template <int LAT, typename S>
 __device__ __forceinline__ void adj_dirichlet_item(const Geom& G, const Band& B, const double* __restrict__ Ub,
                                                    const double* __restrict__ Ub1, const CT<S>* __restrict__ lnext,
-                                                   double* lU, RT<S>* lUr, RT<S>* Y0, int tid)
+                                                   double* lU, RT<S>* lUr, RT<S>* Y0, int u)
 {
-    using L = Lat<LAT>;
-    const int u = tid >> 2, k = tid & 3;
-    if (u >= B.n_unk) return;
-    if (k == 0) {
+    CT<S> d[4];
+    dirichlet_part<LAT, S>(G, B.ud[u], Ub1 + 4LL * u, lnext, 0, d);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) Y0[4LL * u + m] = RT<S>(Ub[4LL * u + m]);
+    for (int k = 0; k < 4; ++k) {
+        Y0[4LL * u + k] = RT<S>(Ub[4LL * u + k]);
+        if (!Lat<LAT>::THERMAL && k == 3) continue;
+        const double v = lU[4LL * u + k] + double(d[k]);
+        lU[4LL * u + k] = v;
+        lUr[4LL * u + k] = RT<S>(v);
     }
-    if (!L::THERMAL && k == 3) return;
-    const double v = lU[4LL * u + k] + double(dirichlet_part<LAT, S>(G, B.ud[u], Ub1 + 4LL * u, lnext, k, 0));
-    lU[4LL * u + k] = v;
-    lUr[4LL * u + k] = RT<S>(v);
 }
 
-// Item (c, k, q) of the corner blocks: node q + 1 of corner c's block.
+// Item (c, q) of the corner blocks: node q + 1 of corner c's block.
 template <int LAT, typename S>
 __device__ __forceinline__ void adj_corner_item(const Geom& G, const Band& B, const AdjState& A,
                                                 const double* __restrict__ Ub1, const CT<S>* __restrict__ lnext,
-                                                int tid)
+                                                int item)
 {
-    using L = Lat<LAT>;
-    const int per = G.M * G.M - 1;
-    const int c = tid / (4 * per), k = (tid / per) % 4, q = tid % per;
+    const int per = G.M * G.M - 1, c = item / per, q = item % per;
     const int u = B.n_unk - 4 + c;
-    A.cpart[tid] = (!L::THERMAL && k == 3)
-                       ? 0.0
-                       : double(dirichlet_part<LAT, S>(G, B.ud[u], Ub1 + 4LL * u, lnext, k, q + 1));
+    CT<S> d[4];
+    dirichlet_part<LAT, S>(G, B.ud[u], Ub1 + 4LL * u, lnext, q + 1, d);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) A.cpart[(c * 4 + k) * per + q] = double(d[k]);
 }
 
 // The other nodes' shares of corner unknown u's block (component k), in
@@ -414,94 +410,107 @@ __device__ __forceinline__ void scatter_ref(const AdjState& A, R* lY, int ref, i
 }
 
 
-// One RK4 stage backwards.  Thread (u, c) evaluates the right-hand side of
-// unknown u (unknown_rhs, charsys.cuh) at the stage field on Dual numbers
-// seeded along inputs 2c, 2c + 1 of: the stage-field values it reads (own,
-// then the two normal and two tangential neighbours; 4 components each),
-// the viscous vector (4) and theta = (alpha_T, beta_P, P_inf - c_s^2 rho0 of
-// its side, alpha_V, t_inf), and adds lambda_k^T dk/dinput to the adjoint of
-// each input.  lambda_k of stage s: U(t+1) = U + (k0 + 2 k1 + 2 k2 + k3)/6,
-// Y1 = U + k0/2, Y2 = U + k1/2, Y3 = U + k2.
+// apply_S (charsys.cuh) backwards: the covector ob of S v adds to the
+// adjoints vb of v and to those of the entries r, a (thermal) or h.
+template <bool TH, typename R>
+__device__ __forceinline__ void adj_apply_S(const CharSys<R>& C, const R* v, const R* ob, R* vb, CharSys<R>& Cb)
+{
+    if (TH) {
+        const R s = ob[2] + ob[3], rvb = s - R(2) * ob[0], avb = ob[3] - ob[2];
+        vb[0] += R(0.25) * C.r * rvb;
+        Cb.r += R(0.25) * v[0] * rvb;
+        vb[3] += R(0.25) * (s + R(2) * ob[0]);
+        vb[1] += C.a * avb;
+        Cb.a += v[1] * avb;
+    } else {
+        const R hvb = ob[2] - ob[0];
+        vb[0] += R(0.5) * (ob[0] + ob[2]);
+        vb[1] += C.h * hvb;
+        Cb.h += v[1] * hvb;
+    }
+    vb[2] += ob[1];
+}
+
+// One RK4 stage backwards, item u: the right-hand side of unknown u
+// (unknown_rhs, charsys.cuh) evaluated at the stage field and run backwards
+// from lambda_k to the stage-field values it reads (own, then the two normal
+// and two tangential neighbours), the viscous vector and theta = (alpha_T,
+// beta_P, P_inf - c_s^2 rho0 of its side, alpha_V, t_inf).  lambda_k of stage s:
+// U(t+1) = U + (k0 + 2 k1 + 2 k2 + k3)/6, Y1 = U + k0/2, Y2 = U + k1/2,
+// Y3 = U + k2.
+//
+// By hand: on forward derivatives along the 29 inputs an unknown took eight
+// threads of four directions each, about 30 times the arithmetic, and
+// k_adj_band 128 us a step (D2Q37 512x256, FP32), now 64 us.
 template <int LAT, typename S>
 __device__ __forceinline__ void adj_vjp_item(const Geom& G, const Band& B, const AdjState& A,
                                              const RT<S>* __restrict__ stU, const RT<S>* __restrict__ stU1,
-                                             int stage, int tid, double (&th)[5])
+                                             int stage, int u, double (&th)[5])
 {
     using R = RT<S>;
-    using T8 = Dual<R, kChunk>;
-    const int u = tid / kRhsChunks, c = tid % kRhsChunks;
-    if (u < B.n_unk) {
-        const UDesc D = B.ud[u];
-        const bool corner = D.kind >= 4;
-        UDesc Dl = D;
-        int ref[5] = {u, 0, 0, 0, 0}, nr;
-        if (corner) {
-            ref[1] = D.nb[0]; ref[2] = D.nb[1];
-            Dl.nb[0] = 1; Dl.nb[1] = 2;
-            nr = 3;
-        } else {
-            if (D.j == B.M) {
-                ref[1] = D.nb[1]; ref[2] = D.nb[2];
-                Dl.nb[1] = 1; Dl.nb[2] = 2;
-            } else {
-                ref[1] = D.nb[0]; ref[2] = D.nb[1];
-                Dl.nb[0] = 1; Dl.nb[1] = 2;
-            }
-            ref[3] = D.nb[4]; ref[4] = D.nb[5];
-            Dl.nb[4] = 3; Dl.nb[5] = 4;
-            nr = 5;
-        }
-        const R frac = stage == 0 ? R(0) : (stage == 3 ? R(1) : R(0.5));
-        CtxT<R> Xr;
-        Xr.Y = static_cast<const R*>(A.Y[stage]);
-        Xr.St = stU;
-        Xr.St1 = stU1;
-        Xr.frac = frac;
-        auto seed = [&](T8& v, int j) {
-            if (j / kChunk == c) v.d[j % kChunk] = R(1);
-        };
-        T8 Yl[20];
+    constexpr bool TH = Lat<LAT>::THERMAL;
+    const UDesc D = B.ud[u];
+    const int kind = D.kind;
+    const bool corner = kind >= 4, outer = corner || D.j == B.M;
+    const R kr = bconst<R>(B.kR, B.kR_f), rho0 = bconst<R>(G.rho0, G.rho0_f), cs2 = R(Lat<LAT>::CS2);
+    CtxT<R> X;
+    X.Y = static_cast<const R*>(A.Y[stage]);
+    X.St = stU;
+    X.St1 = stU1;
+    X.frac = stage == 0 ? R(0) : (stage == 3 ? R(1) : R(0.5));
+    // own value, normal and tangential neighbours
+    int ref[5] = {u, corner ? D.nb[0] : D.j == B.M ? D.nb[1] : D.nb[0], corner ? D.nb[1] : D.j == B.M ? D.nb[2] : D.nb[1],
+                  D.nb[4], D.nb[5]};
+    R v[5][4];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            R v[4] = {R(0), R(0), R(0), R(0)};
-            if (k < nr) fetch(Xr, ref[k], v);
+    for (int k = 0; k < 3; ++k) fetch_local(X, ref[k], kind, kr, v[k]);
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                Yl[4 * k + m] = T8(v[m]);
-                seed(Yl[4 * k + m], 4 * k + m);
-            }
-        }
-        T8 Vd[4];
+    for (int k = 3; k < 5; ++k) {
+        v[k][0] = v[k][1] = v[k][2] = v[k][3] = R(0);
+        if (!corner) fetch_local(X, ref[k], kind, kr, v[k]);
+    }
+    const R *U = v[0], *Up = v[3], *Um = v[4];
+    const R cn = corner ? bconst<R>(B.kC, B.kC_f) : R(0.5);
+    R dUn[4], TT[4] = {0, 0, 0, 0}, VV[4] = {0, 0, 0, 0}, dP = 0;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) dUn[m] = cn * (outer ? R(3) * U[m] - R(4) * v[1][m] + v[2][m] : v[1][m] - v[2][m]);
+    const CharSys<R> C = char_sys_r<TH, R>(B, rho0, U);
+    const R ut = U[2], d_un = R(0.5) * (Up[1] - Um[1]), d_ut = R(0.5) * (Up[2] - Um[2]);
+    R d_rhoT = 0;                       // d rho/dt on D2Q9
+    if (!corner) {
+        d_rhoT = TH ? R(0.5) * ((Up[0] + rho0 * Up[3] + Up[0] * Up[3]) - (Um[0] + rho0 * Um[3] + Um[0] * Um[3]))
+                    : R(0.5) * (Up[0] - Um[0]);
+        TT[0] = R(-0.5) * ((rho0 + Up[0]) * Up[2] - (rho0 + Um[0]) * Um[2]);
+        TT[1] = -ut * d_un;
+        TT[2] = -cs2 * C.irho * d_rhoT - ut * d_ut;
+        if (TH) TT[3] = R(-0.5) * ((R(1) + Up[3]) * Up[2] - (R(1) + Um[3]) * Um[2]);
+        dP = (TH ? cs2 * (U[0] + rho0 * U[3] + U[0] * U[3]) : cs2 * U[0]) - relax_value<R>(A, 4 + kind);
         const R* Vu = static_cast<const R*>(A.V) + 4LL * u;
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            Vd[m] = T8(Vu[m]);
-            seed(Vd[m], 20 + m);
-        }
-        Relax<T8> P;
-        P.alpha_T = T8(relax_value<R>(A, 0));
-        P.beta_P = T8(relax_value<R>(A, 1));
-        P.t_inf = T8(relax_value<R>(A, 2));
-        P.alpha_V = T8(relax_value<R>(A, 3));
+        for (int m = 0; m < 4; ++m) VV[m] = Vu[m];
+    }
+    const int scheme = corner ? int(SCH_LODI) : B.scheme[kind], mask = A.mask[u];
+    const bool cbc = scheme == SCH_CBC || scheme == SCH_CBC_RELAX;
+    const R aT = relax_value<R>(A, 0), bP = relax_value<R>(A, 1), ti = relax_value<R>(A, 2), aV = relax_value<R>(A, 3);
+    R sd[4], st[4], sv[4], w[4];
+    apply_S<TH>(C, dUn, sd);
+    apply_S<TH>(C, TT, st);
+    apply_S<TH>(C, VV, sv);
+    // the weights of S T, S V and beta (P - P_inf) in an incoming wave
+    const R fT = scheme == SCH_CBC ? R(1) : scheme == SCH_CBC_RELAX ? R(1) - aT : scheme == SCH_LODI_RELAX ? -aT : R(0);
+    const R fV = scheme == SCH_CBC ? R(1) : scheme == SCH_CBC_RELAX ? R(1) - aV : R(0);
+    const bool relax = scheme == SCH_LODI_RELAX || scheme == SCH_CBC_RELAX;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) P.pdev[q] = T8(relax_value<R>(A, 4 + q));
-        seed(P.alpha_T, 24);
-        seed(P.beta_P, 25);
-        if (!corner) {
-            T8& pd = D.kind == 0 ? P.pdev[0] : D.kind == 1 ? P.pdev[1] : D.kind == 2 ? P.pdev[2] : P.pdev[3];
-            seed(pd, 26);
-        }
-        seed(P.alpha_V, 27);
-        seed(P.t_inf, 28);
-        CtxT<T8> Xl;
-        Xl.Y = Yl;
-        Xl.St = Xl.St1 = nullptr;
-        Xl.frac = T8(frac);
-        T8 k[4];
-        unknown_rhs<LAT, T8>(G, B, P, Xl, Dl, 0, Vd, A.mask[u], k);
-        const R cs = (stage == 0 || stage == 3) ? R(1.0 / 6.0) : R(1.0 / 3.0);
-        const R ch = stage == 2 ? R(1) : R(0.5);
-        R lk[4];
+    for (int i = 0; i < 4; ++i) {
+        const bool acoustic = TH ? i >= 2 : i != 1;
+        if (!TH && i == 3) w[i] = R(0);
+        else if (!((mask >> i) & 1)) w[i] = C.lam[i] * sd[i];
+        else w[i] = fT * st[i] + fV * sv[i] + (relax ? aT * ti + (acoustic ? bP * dP : R(0)) : R(0));
+    }
+    // lambda_k, in the local frame (the frames are orthonormal)
+    R kb[4], kl[4];
+    {
+        const R cs = (stage == 0 || stage == 3) ? R(1.0 / 6.0) : R(1.0 / 3.0), ch = stage == 2 ? R(1) : R(0.5);
         R* lUr = static_cast<R*>(A.lUr) + 4LL * u;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -510,86 +519,217 @@ __device__ __forceinline__ void adj_vjp_item(const Geom& G, const Band& B, const
                 // the corner block's other nodes (adj_corner_item) join here;
                 // the stages after this one read the rounded sum
                 lu = R(A.lU[4LL * u + m] + corner_share(G, B, A, u, m));
-                if (c == 0) lUr[m] = lu;
+                lUr[m] = lu;
             }
-            lk[m] = cs * lu;
-            if (stage < 3) lk[m] += ch * static_cast<const R*>(A.lY[stage + 1])[4LL * u + m];
+            kl[m] = cs * lu;
+            if (stage < 3) kl[m] += ch * static_cast<const R*>(A.lY[stage + 1])[4LL * u + m];
         }
-        R* lY = static_cast<R*>(A.lY[stage]);
+        to_local(kind, kr, kl, kb);
+    }
+    // backwards: S^-1 and the waves
+    CharSys<R> Cb;
+    Cb.rho = Cb.irho = Cb.r = Cb.ir = Cb.a = Cb.b = Cb.h = Cb.csr = R(0);
+    R wb[4], sdb[4], stb[4], svb[4], lsum = 0, lc = 0, dPb = 0;
+    if (TH) {
+        const R o0 = -kb[0], o1 = -kb[1], o3 = -kb[3];
+        Cb.ir = o0 * (w[2] + w[3] - w[0]);
+        Cb.b = o1 * (w[3] - w[2]);
+        wb[0] = o3 - o0 * C.ir;
+        wb[2] = o3 + o0 * C.ir - o1 * C.b;
+        wb[3] = o3 + o0 * C.ir + o1 * C.b;
+    } else {
+        const R o0 = -kb[0], o1 = -kb[1];
+        Cb.csr = o1 * (w[2] - w[0]);
+        wb[0] = o0 - o1 * C.csr;
+        wb[2] = o0 + o1 * C.csr;
+        wb[3] = R(0);
+    }
+    wb[1] = -kb[2];
+    R tb[5] = {0, 0, 0, 0, 0};
 #pragma unroll
-        for (int d = 0; d < kChunk; ++d) {
-            const int j = kChunk * c + d;
-            if (j >= kRhsInputs) break;
-            R g = R(0);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) g += lk[m] * k[m].d[d];
-            if (g == R(0)) continue;
-            if (j < 20) {
-                if (j / 4 < nr) scatter_ref<R>(A, lY, ref[j / 4], j % 4, frac, g);
-            } else if (j < 24) {
-                static_cast<R*>(A.lV)[4LL * u + (j - 20)] += g;      // one thread per (u, j)
-            } else {
-                th[j - 24] += double(g);
+    for (int i = 0; i < 4; ++i) {
+        sdb[i] = stb[i] = svb[i] = R(0);
+        if (!TH && i == 3) continue;
+        const bool acoustic = TH ? i >= 2 : i != 1;
+        if (!((mask >> i) & 1)) {
+            const R l = wb[i] * sd[i];
+            sdb[i] = wb[i] * C.lam[i];
+            lsum += l;
+            if (TH && i == 2) lc -= l;
+            if (TH && i == 3) lc += l;
+            continue;
+        }
+        stb[i] = fT * wb[i];
+        svb[i] = fV * wb[i];
+        if (relax) {
+            tb[0] += wb[i] * (ti - st[i]);
+            tb[4] += wb[i] * aT;
+            if (scheme == SCH_CBC_RELAX) tb[3] -= wb[i] * sv[i];
+            if (acoustic) {
+                tb[1] += wb[i] * dP;
+                dPb += wb[i] * bP;
             }
         }
     }
+    tb[2] = -dPb;
+    R dUb[4] = {0, 0, 0, 0}, TTb[4], VVb[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) TTb[m] = VVb[m] = cbc ? kb[m] : R(0);
+    adj_apply_S<TH>(C, dUn, sdb, dUb, Cb);
+    adj_apply_S<TH>(C, TT, stb, TTb, Cb);
+    adj_apply_S<TH>(C, VV, svb, VVb, Cb);
+    // the stage field: own value and neighbours
+    R vb[5][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const R d = cn * dUb[m];
+        vb[0][m] = outer ? R(3) * d : R(0);
+        vb[1][m] = outer ? R(-4) * d : d;
+        vb[2][m] = outer ? d : -d;
+        vb[3][m] = vb[4][m] = R(0);
+    }
+    R irb = Cb.irho;
+    vb[0][1] += lsum;
+    if (!corner) {
+        const R t0 = R(-0.5) * TTb[0], t1 = R(-0.5) * ut * TTb[1], t2 = R(-0.5) * ut * TTb[2],
+                h = R(-0.5) * cs2 * C.irho * TTb[2];
+        irb -= cs2 * d_rhoT * TTb[2];
+        vb[0][2] -= TTb[1] * d_un + TTb[2] * d_ut;
+        vb[3][0] += t0 * Up[2];
+        vb[4][0] -= t0 * Um[2];
+        vb[3][1] += t1;
+        vb[4][1] -= t1;
+        vb[3][2] += t0 * (rho0 + Up[0]) + t2;
+        vb[4][2] -= t0 * (rho0 + Um[0]) + t2;
+        if (TH) {
+            const R t3 = R(-0.5) * TTb[3];
+            vb[3][0] += h * (R(1) + Up[3]);
+            vb[4][0] -= h * (R(1) + Um[3]);
+            vb[3][3] += h * (rho0 + Up[0]) + t3 * Up[2];
+            vb[4][3] -= h * (rho0 + Um[0]) + t3 * Um[2];
+            vb[3][2] += t3 * (R(1) + Up[3]);
+            vb[4][2] -= t3 * (R(1) + Um[3]);
+            vb[0][0] += cs2 * dPb * (R(1) + U[3]);
+            vb[0][3] += cs2 * dPb * (rho0 + U[0]);
+        } else {
+            vb[3][0] += h;
+            vb[4][0] -= h;
+            vb[0][0] += cs2 * dPb;
+        }
+    }
+    // the characteristic system (char_sys_r)
+    R rhob = 0;
+    if (TH) {
+        const R kA = bconst<R>(B.kA, B.kA_f), kB = bconst<R>(B.kB, B.kB_f);
+        const R tht = R(1) + U[3], isth = R(1) / sqrt(tht);
+        const R isb = kB * Cb.b + R(2) * C.rho * isth * Cb.ir;
+        const R sb = kA * Cb.a + kB * lc - isth * isth * isb;
+        rhob = isth * isth * Cb.ir;
+        irb += tht * Cb.r;
+        vb[0][3] += C.irho * Cb.r + R(0.5) * isth * sb;
+    } else {
+        rhob = bconst<R>(B.ihcs, B.ihcs_f) * Cb.h;
+        irb += bconst<R>(B.cs, B.cs_f) * Cb.csr;
+    }
+    vb[0][0] += rhob - C.irho * C.irho * irb;
+    R* lY = static_cast<R*>(A.lY[stage]);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        if (k >= 3 && corner) break;
+        R g[4];
+        to_lab(kind, kr, vb[k], g);
+#pragma unroll
+        for (int m = 0; m < (TH ? 4 : 3); ++m)
+            if (g[m] != R(0)) scatter_ref<R>(A, lY, ref[k], m, X.frac, g[m]);
+    }
+    if (!corner) {
+        R* lV = static_cast<R*>(A.lV) + 4LL * u;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) lV[m] += VVb[m];        // one thread per unknown
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+        if (tb[q] != R(0)) th[q] += double(tb[q]);
 }
 
 // The mesoscopic viscous vector of side unknown u (vis_meso, Eqs. LaplaceU,
-// LaplaceT) backwards to its stencil's strip values of time t: thread (u, c)
-// takes inputs 2c, 2c + 1 of (5 moments, u_x, u_y) per stencil node, then
-// drho of the first node.
+// LaplaceT) backwards to its stencil's strip values of time t: per node the
+// 5 moments and u_x, u_y, and drho of the first node.
 template <int LAT, typename S>
 __device__ __forceinline__ void adj_vis_meso_item(const Geom& G, const Band& B, const AdjState& A,
-                                                  const RT<S>* __restrict__ stU, const RT<S>* __restrict__ stN, int tid)
+                                                  const RT<S>* __restrict__ stU, const RT<S>* __restrict__ stN, int u)
 {
-    using Lt = Lat<LAT>;
     using R = RT<S>;
-    using T8 = Dual<R, kChunk>;
-    const int u = tid / kMesoChunks, c = tid % kMesoChunks;
-    if (u >= B.n_unk) return;
+    constexpr bool TH = Lat<LAT>::THERMAL;
+    constexpr R ics2 = R(1.0 / Lat<LAT>::CS2);
     const UDesc D = B.ud[u];
     if (D.kind >= 4) return;
     const R* lV = static_cast<const R*>(A.lV) + 4LL * u;
-    if (lV[0] == R(0) && lV[1] == R(0) && lV[2] == R(0) && lV[3] == R(0)) return;
-    T8 SU[5 * 4], SN[5 * 5];
-    UDesc Dl = D;
+    const R l1 = lV[1], l2 = lV[2], l3 = TH ? lV[3] : R(0);
+    if (l1 == R(0) && l2 == R(0) && l3 == R(0)) return;
+    const int an = D.kind < 2 ? 0 : 1, at = 1 - an;
+    const R sn = (D.kind == 0 || D.kind == 2) ? R(-1) : R(1);
+    // in the local frame: sigma'_nn, sigma'_nt, sigma'_tt, q_n, q_t, u_n, u_t
+    R h[5][7];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        const int sl = D.vs[k];
-        Dl.vs[k] = k;
+        const R* n = stN + 5LL * D.vs[k];
+        const R* U = stU + 4LL * D.vs[k];
+        h[k][0] = an == 0 ? n[0] : n[2];
+        h[k][1] = sn * n[1];
+        h[k][2] = an == 0 ? n[2] : n[0];
+        h[k][3] = sn * n[3 + an];
+        h[k][4] = n[3 + at];
+        h[k][5] = sn * U[1 + an];
+        h[k][6] = U[1 + at];
+    }
+    // d_n f = sum dn[k] f_k; d_t f likewise, central or one-sided
+    const R dn[5] = {R(1.5), R(-2), R(0.5), R(0), R(0)};
+    const R tm = R(0.5) * R(D.tmode);
+    const R dt[5] = {R(3) * tm, R(0), R(0), D.tmode == 0 ? R(0.5) : R(-4) * tm, D.tmode == 0 ? R(-0.5) : tm};
+    auto diff = [&](const R* d, int m) {
+        R v = R(0);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) SU[4 * k + m] = T8(stU[4LL * sl + m]);
-#pragma unroll
-        for (int m = 0; m < 5; ++m) SN[5 * k + m] = T8(stN[5LL * sl + m]);
+        for (int k = 0; k < 5; ++k) v += d[k] * h[k][m];
+        return v;
+    };
+    const R irho = R(1) / (bconst<R>(G.rho0, G.rho0_f) + stU[4LL * D.vs[0]]);
+    const R s1 = diff(dn, 0) + diff(dt, 1), s2 = diff(dn, 1) + diff(dt, 2);
+    R bn[7] = {irho * l1, irho * l2, R(0), R(0), R(0), R(0), R(0)};     // adjoints of d_n h_m
+    R bt[7] = {R(0), irho * l1, irho * l2, R(0), R(0), R(0), R(0)};     // and of d_t h_m
+    R ib = l1 * s1 + l2 * s2;
+    if (TH) {
+        const R c = -irho * ics2 * l3, nu = R(G.tau - 0.5);             // nu / c_s^2 = tau - 1/2
+        bn[3] = c;
+        bt[4] = c;
+        ib -= ics2 * l3 * (diff(dn, 3) + diff(dt, 4));
+        const R e1 = R(2) * nu * l3 * (diff(dn, 5) - diff(dt, 6)), e2 = R(2) * nu * l3 * (diff(dn, 6) + diff(dt, 5));
+        bn[5] = e1;
+        bt[6] = -e1;
+        bn[6] = e2;
+        bt[5] = e2;
     }
 #pragma unroll
-    for (int d = 0; d < kChunk; ++d) {
-        const int j = kChunk * c + d;
-        if (j >= kMesoInputs) break;
-        if (j == 35) { SU[0].d[d] = R(1); continue; }
-        const int k = j / 7, m = j % 7;
-        if (m < 5) SN[5 * k + m].d[d] = R(1);
-        else SU[4 * k + (m - 4)].d[d] = R(1);   // m = 5: u_x, m = 6: u_y
-    }
-    T8 Vo[4];
-    vis_meso<Lt::THERMAL, T8>(G, SU, 4, SN, 5, Dl, Lt::CS2, Vo);
+    for (int k = 0; k < 5; ++k) {
+        R g[7];
 #pragma unroll
-    for (int d = 0; d < kChunk; ++d) {
-        const int j = kChunk * c + d;
-        if (j >= kMesoInputs) break;
-        R g = R(0);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) g += lV[m] * Vo[m].d[d];
-        if (g == R(0)) continue;
-        if (j == 35) {
-            atomicAdd(static_cast<R*>(A.lSt) + 4LL * D.vs[0], g);
-            continue;
+        for (int m = 0; m < 7; ++m) g[m] = dn[k] * bn[m] + dt[k] * bt[m];
+        R* ln = static_cast<R*>(A.lN) + 5LL * D.vs[k];
+        R* lu = static_cast<R*>(A.lSt) + 4LL * D.vs[k];
+        auto add = [](R* p, R v) {
+            if (v != R(0)) atomicAdd(p, v);
+        };
+        add(ln + (an == 0 ? 0 : 2), g[0]);
+        add(ln + 1, sn * g[1]);
+        add(ln + (an == 0 ? 2 : 0), g[2]);
+        if (TH) {
+            add(ln + 3 + an, sn * g[3]);
+            add(ln + 3 + at, g[4]);
+            add(lu + 1 + an, sn * g[5]);
+            add(lu + 1 + at, g[6]);
         }
-        const int k = j / 7, m = j % 7, sl = D.vs[k];
-        if (m < 5) atomicAdd(static_cast<R*>(A.lN) + 5LL * sl + m, g);
-        else atomicAdd(static_cast<R*>(A.lSt) + 4LL * sl + (m - 4), g);
     }
+    atomicAdd(static_cast<R*>(A.lSt) + 4LL * D.vs[0], -irho * irho * ib);
 }
 
 // The "-FD" viscous vector of side unknown u (vis_fd, Sec. 4.2) backwards to
@@ -755,6 +895,9 @@ __global__ void __launch_bounds__(kBandThreads, 2)
     using R = RT<S>;
     cg::grid_group grid = cg::this_grid();
     const int nth = int(gridDim.x * blockDim.x), t0 = int(blockIdx.x * blockDim.x + threadIdx.x);
+    // items of a phase are dealt to the CTAs warp by warp, so that a few
+    // thousand of them (one to an unknown) run on every SM
+    const int w0 = int((threadIdx.x / 32 * gridDim.x + blockIdx.x) * 32 + threadIdx.x % 32);
     const int nu = B.n_unk;
     StageSet Z;
 #pragma unroll
@@ -762,19 +905,17 @@ __global__ void __launch_bounds__(kBandThreads, 2)
     Z.V = A.V;
     Z.mask = A.mask;
     // the corner unknowns, if any, are the last four
-    const int ncp = (nu >= 4 && B.ud[nu - 4].kind == 4) ? 16 * (G.M * G.M - 1) : 0;
-    for (int i = t0; i < 4 * nu + ncp; i += nth) {
-        if (i < 4 * nu) {
-            if (nxt && (i & 3) == 1) {
-                R* y = static_cast<R*>(Zn.Y[0]) + 4LL * (i >> 2);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) y[m] = R(Ubm[4LL * (i >> 2) + m]);
-            }
-            adj_dirichlet_item<LAT, S>(G, B, Ub, Ub1, lnext, A.lU, static_cast<R*>(A.lUr), static_cast<R*>(A.Y[0]), i);
-        } else {
-            adj_corner_item<LAT, S>(G, B, A, Ub1, lnext, i - 4 * nu);
-        }
+    const int ncp = (nu >= 4 && B.ud[nu - 4].kind == 4) ? 4 * (G.M * G.M - 1) : 0;
+    for (int i = w0; i < nu + ncp; i += nth) {
+        if (i < nu) adj_dirichlet_item<LAT, S>(G, B, Ub, Ub1, lnext, A.lU, static_cast<R*>(A.lUr), static_cast<R*>(A.Y[0]), i);
+        else adj_corner_item<LAT, S>(G, B, A, Ub1, lnext, i - nu);
     }
+    if (nxt)
+        for (int i = t0; i < nu; i += nth) {
+            R* y = static_cast<R*>(Zn.Y[0]) + 4LL * i;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) y[m] = R(Ubm[4LL * i + m]);
+        }
     {
         R* z = static_cast<R*>(A.lY[0]);     // lY[0..3] and lV, contiguous
         for (long long i = t0; i < 20LL * nu; i += nth) z[i] = R(0);
@@ -782,21 +923,23 @@ __global__ void __launch_bounds__(kBandThreads, 2)
     grid.sync();
     if (!pre) {
         for (int s = 0; s < 3; ++s) {
-            for (int u = t0; u < nu; u += nth) adj_fwd_item<LAT, S>(G, B, A, Z, stU, stN, stU1, s, u);
+            for (int u = w0; u < nu; u += nth) adj_fwd_item<LAT, S>(G, B, A, Z, stU, stN, stU1, s, u);
             grid.sync();
         }
     }
     double th[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     for (int s = 3; s >= 0; --s) {
-        const int nv = nu * kRhsChunks, nf = (nxt && s > 0) ? nu : 0;
-        for (int i = t0; i < nv + nf; i += nth) {
-            if (i < nv) adj_vjp_item<LAT, S>(G, B, A, stU, stU1, s, i, th);
-            else adj_fwd_item<LAT, S>(G, B, A, Zn, stUm, stNm, stU, 3 - s, i - nv);
+        // whole warps per kind of item: the stage fields from the next
+        // multiple of 32
+        const int nv = (nu + 31) / 32 * 32, nf = (nxt && s > 0) ? nu : 0;
+        for (int i = w0; i < nv + nf; i += nth) {
+            if (i < nu) adj_vjp_item<LAT, S>(G, B, A, stU, stU1, s, i, th);
+            else if (i >= nv) adj_fwd_item<LAT, S>(G, B, A, Zn, stUm, stNm, stU, 3 - s, i - nv);
         }
         grid.sync();
     }
     if (B.viscous == VIS_MESO) {
-        for (int i = t0; i < nu * kMesoChunks; i += nth) adj_vis_meso_item<LAT, S>(G, B, A, stU, stN, i);
+        for (int i = w0; i < nu; i += nth) adj_vis_meso_item<LAT, S>(G, B, A, stU, stN, i);
     } else if (B.viscous == VIS_FD) {
         for (int i = t0; i < nu * kFdChunks; i += nth) adj_vis_fd_item<LAT, S>(G, B, A, stU, i);
     }
@@ -1008,9 +1151,9 @@ int adj_step_t(const Geom& G, const Export& E, const Band& B, const Region& bulk
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_band<LAT, S>, kBandThreads, 0) != cudaSuccess ||
                 per_sm < 1)
                 return -1;
-            // two CTAs per SM at most: more measured slower (longer grid
-            // barriers, less room for the kernels on the other streams)
-            grid_ctas = std::min(per_sm, 2) * sms;
+            // one CTA per SM: more make the grid barriers longer and leave
+            // less room for the kernels on the other streams
+            grid_ctas = sms;
         }
         const double* a_Ub = Ub;
         const double* a_Ub1 = Ub1;
