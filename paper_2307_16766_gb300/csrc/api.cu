@@ -1843,8 +1843,12 @@ int batch_issue_step(lbm_batch* b, int par, cudaStream_t s0, bool with_inflow)
 }
 
 // Pick the persistent bulk kernel's CTAs per SM for each group: the fastest
-// of 1..5 over three timed launches each (the launches rewrite the new
-// buffer from the current one, which the following step rewrites again).
+// of 1..5 over three timed steps each (they rewrite the new buffers and the
+// new boundary state from the current ones, which the following step rewrites
+// again).  Whole steps, not the bulk kernel alone: with five CTAs per SM it is
+// fastest by itself, with three or four it leaves the band tiles beside it
+// room (96 runs of 128^2 to 512^2, FP32: 40 steps with their fields 29.6 ms
+// with five, 28.0 ms with three or four).
 int batch_autotune(lbm_batch* b)
 {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1858,19 +1862,16 @@ int batch_autotune(lbm_batch* b)
         if (!best) {
             float best_ms = 1e30f;
             for (int m = 1; m <= 5; ++m) {
-                const int grid = b->nsm * m;
-                launch_bulk_persistent(g.lattice, g.storage, g.bulk, int(g.members.size()), g.total_items, par,
-                                       grid, g.queue, b->stream);        // warm-up
+                g.grid = b->nsm * m;
+                int rc = batch_issue_step(b, par, b->stream, false);     // warm-up
                 cudaEventRecord(e0, b->stream);
-                for (int r = 0; r < 3; ++r)
-                    launch_bulk_persistent(g.lattice, g.storage, g.bulk, int(g.members.size()), g.total_items,
-                                           par, grid, g.queue, b->stream);
+                for (int r = 0; r < 3 && rc == LBM_OK; ++r) rc = batch_issue_step(b, par, b->stream, false);
                 cudaEventRecord(e1, b->stream);
                 e = cudaEventSynchronize(e1);
-                if (e != cudaSuccess) {
+                if (rc != LBM_OK || e != cudaSuccess) {
                     cudaEventDestroy(e0);
                     cudaEventDestroy(e1);
-                    return batch_fail(b, e, "autotune");
+                    return rc != LBM_OK ? rc : batch_fail(b, e, "autotune");
                 }
                 float ms = 0.0f;
                 cudaEventElapsedTime(&ms, e0, e1);
