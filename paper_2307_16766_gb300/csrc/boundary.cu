@@ -16,6 +16,7 @@
 // and t + 1 (interpolated linearly at the stage time, Sec. 3.3).
 #include "charsys.cuh"
 #include "ff.cuh"
+#include "fix64.cuh"
 
 #include <algorithm>
 #include <cooperative_groups.h>
@@ -651,19 +652,17 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     auto pull_t1 = [&](int k, const StripNode& N) {
         C g[L::Q];
         pull_plain<LAT, S, C>(G, O, fin, N.x, N.y, g);
-        if (Store<S>::SCALED) {
-#pragma unroll
-            for (int i = 0; i < L::Q; ++i) g[i] *= C(L::w(i));
-        }
+        // sums and collision on the integer pipe (fix64.cuh) where the numbers
+        // are in its range
         Moments<LAT, C> m;
+        auto get = [&](int i) { return g[i]; };
+        const int emax = fx_block<LAT>(get);
+        if (!emax || !fx_moments<LAT>(get, G.rho0, REF ? G.ref : 0, G.uref[0], G.uref[1], m))
+            m = moments_G<LAT, C, REF>(G, g);
         if (N.fx >= 0) {
             S* fx = Fx + N.fx * L::Q;
-            m = collide<LAT, C, REF>(G, g, [&](int i, C v) {
-                if (Store<S>::SCALED) v *= C(1.0 / L::w(i));
-                Store<S>::put(fx + i, v);
-            });
-        } else {
-            m = moments_G<LAT, C, REF>(G, g);
+            auto put = [&](int i, C v) { fx[i] = v; };
+            if (m.ref || !emax || !fx_relax<LAT>(m, G.omega, get, put)) collide_given<LAT, C>(G, m, get, put);
         }
         const R U1[4] = {R(m.s0), R(m.ux), R(m.uy), R(m.dT)};
 #pragma unroll
@@ -674,7 +673,14 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
             for (int c = 0; c < 4; ++c) u[c] = U1[c];
             if (N.flags & kSNNeq) {     // a node of the mesoscopic stencil
                 R N1[5];
-                neq_moments<LAT, C, R>(g, m, R(1) - R(0.5) * omega_of<R>(G), N1);
+                const R fac = R(1) - R(0.5) * omega_of<R>(G);
+                if (emax) {
+                    R pxy, dxy, pxx, pyy, rx, ry;
+                    fx_neq_sums<LAT>(get, emax, pxy, dxy, pxx, pyy, rx, ry);
+                    neq_close<LAT, C, R>(m, fac, N1, pxy, dxy, pxx, pyy, rx, ry);
+                } else {
+                    neq_moments<LAT, C, R>(g, m, fac, N1);
+                }
                 R* q = static_cast<R*>(E.stripN) + ((long long)(par_t ^ 1) * E.nslots + N.gslot) * 5;
 #pragma unroll
                 for (int c = 0; c < 5; ++c) q[c] = N1[c];

@@ -18,6 +18,7 @@
 // FP32; the FP64 path in FP64.
 #include "collide.cuh"
 #include "ff.cuh"
+#include "fix64.cuh"
 
 #include <utility>
 
@@ -134,6 +135,53 @@ __device__ __forceinline__ void gather_staged(C* g, const S* sb, int t,
      ...);
 }
 
+// FP64 storage held against w rho0: the collision on the integer pipe
+// (fix64.cuh), its populations read from the staging buffer as needed.
+template <typename S, bool REF>
+constexpr bool bulk_fixed() { return sizeof(S) == 8 && !REF; }
+
+// The staged value of velocity i for the thread whose column sb points to.
+template <int LAT, typename S>
+struct Slots {
+    int at[Lat<LAT>::Q];
+    constexpr Slots() : at()
+    {
+        for (int i = 0; i < Lat<LAT>::Q; ++i) at[i] = Stage<LAT, S>::elem(i) + Stage<LAT, S>::H - Lat<LAT>::cx(i);
+    }
+};
+
+// The FP64 form, for numbers out of the fixed-point range.
+template <int LAT>
+__device__ __noinline__ void collide_wide(const Geom& G, const double* sb, double* out, const int* st, int plane)
+{
+    constexpr Slots<LAT, double> slot{};
+    double g[Lat<LAT>::Q];
+#pragma unroll
+    for (int i = 0; i < Lat<LAT>::Q; ++i) g[i] = sb[slot.at[i]];
+    collide<LAT, double, false>(G, g, [&](int i, double v) { out[st ? st[i] : Lat<LAT>::plane_of(i) * plane] = v; });
+}
+
+// Plainly pulled populations into the thread's own staging slots.
+template <int LAT, typename S>
+__device__ __forceinline__ void put_staged(const S* g, S* sb)
+{
+    constexpr Slots<LAT, S> slot{};
+#pragma unroll
+    for (int i = 0; i < Lat<LAT>::Q; ++i) sb[slot.at[i]] = g[i];
+}
+
+// One staged node; st: output offsets (null: planes of `plane` elements).
+template <int LAT>
+__device__ __forceinline__ void collide_staged(const Geom& G, const double* sb, double* out, const int* st, int plane)
+{
+    constexpr Slots<LAT, double> slot{};
+    auto get = [&](int i) { return sb[slot.at[i]]; };
+    Moments<LAT, double> m;
+    if (!fx_moments<LAT>(get, G.rho0, 0, 0.0, 0.0, m) ||
+        !fx_relax<LAT>(m, G.omega, get, [&](int i, double v) { out[st ? st[i] : Lat<LAT>::plane_of(i) * plane] = v; }))
+        collide_wide<LAT>(G, sb, out, st, plane);
+}
+
 // Pull-stream result g of node (x, y) -> moments, BGK collision (Eq. bgk)
 // and post-collision store.
 template <int LAT, typename S, typename C, bool REF>
@@ -206,6 +254,7 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
     for (int r = 0; r < ROWS; ++r) {
         const int y = yb + r;
         if (y >= R.y1) break;
+        constexpr bool FIXED = bulk_fixed<S, REF>();
         C g[Q];
         if (staged(y)) {
             if (!wait_tx(&bar[r], status, G.wait_ns)) {
@@ -216,13 +265,19 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
                 return;
             }
             if (!valid) continue;
-            gather_staged<LAT, S, C>(g, reinterpret_cast<const S*>(smem_raw + r * BX::TOTAL), threadIdx.x,
-                                     std::make_integer_sequence<int, Q>{});
+            if constexpr (!FIXED)
+                gather_staged<LAT, S, C>(g, reinterpret_cast<const S*>(smem_raw + r * BX::TOTAL), threadIdx.x,
+                                         std::make_integer_sequence<int, Q>{});
         } else {
             if (!valid) continue;
             pull_plain<LAT, S, C>(G, O, fin, x, y, g);
+            if constexpr (FIXED)
+                put_staged<LAT, S>(g, reinterpret_cast<S*>(smem_raw + r * BX::TOTAL) + threadIdx.x);
         }
-        collide_store<LAT, S, C, REF>(G, O, fout, x, y, g);
+        if constexpr (FIXED)
+            collide_staged<LAT>(G, reinterpret_cast<const double*>(smem_raw + r * BX::TOTAL) + threadIdx.x,
+                                reinterpret_cast<double*>(fout) + (y * G.nxp + x), O.st, 0);
+        else collide_store<LAT, S, C, REF>(G, O, fout, x, y, g);
     }
 }
 
@@ -237,10 +292,11 @@ __device__ __forceinline__ void bulk_end(int chain)
         pdl_wait();
 }
 
+// (FP64: three CTAs per SM, all that 168 registers of D2Q37 leave room for.)
 template <int LAT, typename S>
-__global__ void __launch_bounds__(kBulkThreads)
-    k_bulk(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
-           S* __restrict__ fout, int* status, int chain)
+__global__ void __launch_bounds__(kBulkThreads, sizeof(S) == 8 ? 3 : 0)
+    k_bulk(const __grid_constant__ Maps tm, const __grid_constant__ Geom G, const __grid_constant__ Offsets O, Region R,
+           const S* __restrict__ fin, S* __restrict__ fout, int* status, int chain)
 {
     pdl_trigger();
     bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status, chain);
@@ -353,11 +409,14 @@ __global__ void __launch_bounds__(kBulkThreads)
             if (stage) phase1 ^= 1u;
             else phase0 ^= 1u;
             ok = __syncthreads_and(ok);     // one decision for the whole CTA
-            if (ok && valid)
-                gather_staged<LAT, S, C>(g, reinterpret_cast<const S*>(smem_raw + stage * BX::TOTAL),
-                                         threadIdx.x, std::make_integer_sequence<int, L::Q>{});
+            if constexpr (!bulk_fixed<S, false>())
+                if (ok && valid)
+                    gather_staged<LAT, S, C>(g, reinterpret_cast<const S*>(smem_raw + stage * BX::TOTAL),
+                                             threadIdx.x, std::make_integer_sequence<int, L::Q>{});
         } else if (valid) {
             pull_plain_planes<LAT, S, C>(R.G, static_cast<const S*>(R.f[par]), x, cur.y, g);
+            if constexpr (bulk_fixed<S, false>())
+                put_staged<LAT, S>(g, reinterpret_cast<S*>(smem_raw + stage * BX::TOTAL) + threadIdx.x);
         }
         if (!ok) {
             // a copy never completed: wait (bounded) for the one in flight
@@ -371,6 +430,9 @@ __global__ void __launch_bounds__(kBulkThreads)
             auto put = [&](int i, C v) { Store<S>::put(out + L::plane_of(i) * plane, v); };
             // runs of a batch hold the plain shift (lbm_batch_create)
             if constexpr (Store<S>::SCALED) collide_scaled<LAT, false>(R.G, g, put);
+            else if constexpr (bulk_fixed<S, false>())
+                collide_staged<LAT>(R.G, reinterpret_cast<const double*>(smem_raw + stage * BX::TOTAL) + threadIdx.x,
+                                    reinterpret_cast<double*>(out), nullptr, plane);
             else collide<LAT, C, false>(R.G, g, put);
         }
         __syncthreads();                    // stage buffer read by all before its reuse
@@ -421,14 +483,21 @@ __global__ void k_init(Geom G, Export E, const double* __restrict__ rho,
         mc.vx = C(m.ux - stored_ref<S>(G, 0));
         mc.vy = C(m.uy - stored_ref<S>(G, 1));
     }
-    C geq[L::Q];
-    equilibrium<LAT, C>(mc, geq);
     S* out = f + (long long)y * G.nxp + x;
+    bool done = false;
+    if constexpr (sizeof(S) == 8)       // FP64 on the integer pipe, as the bulk update
+        if (!G.ref) done = fx_equilibrium<LAT>(mc, mc.rho * mc.ux, mc.rho * mc.uy, [&](int i, FxConst w, long long x, int e) {
+                out[L::plane_of(i) * G.plane] = fx_scaled(x, w, e);
+            });
+    if (!done) {
+        C geq[L::Q];
+        equilibrium<LAT, C>(mc, geq);
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        C v = geq[i];
-        if (Store<S>::SCALED) v *= C(1.0 / L::w(i));
-        Store<S>::put(out + (long long)L::plane_of(i) * G.plane, v);
+        for (int i = 0; i < L::Q; ++i) {
+            C v = geq[i];
+            if (Store<S>::SCALED) v *= C(1.0 / L::w(i));
+            Store<S>::put(out + (long long)L::plane_of(i) * G.plane, v);
+        }
     }
     // strips of time 0 (parity 0): U0 and zero non-equilibrium moments
     const int dd[4] = {x - G.M, G.nx - 1 - G.M - x, y - G.M, G.ny - 1 - G.M - y};
@@ -523,7 +592,7 @@ __global__ void __launch_bounds__(kBulkThreads) k_macros(Geom G, const S* __rest
     const int y = blockIdx.y;
     if (x >= G.nx) return;
     const S* in = f + (long long)y * G.nxp + x;
-    double U[4];
+    double U[4] = {0.0, 0.0, 0.0, 0.0};
     auto finite = [&]() { return isfinite(U[0]) && isfinite(U[1]) && isfinite(U[2]) && isfinite(U[3]); };
     if constexpr (sizeof(typename Store<S>::C) == 4) {
         float h[L::Q];
@@ -532,7 +601,18 @@ __global__ void __launch_bounds__(kBulkThreads) k_macros(Geom G, const S* __rest
         macros_ff<LAT, S>(G, h, U);
         if (!finite()) macros_wide<LAT, S>(G, in, U);   // beyond the float range
     } else {
-        macros_wide<LAT, S>(G, in, U);
+        double g[L::Q];
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) g[i] = Store<S>::load(in + (long long)L::plane_of(i) * G.plane);
+        Moments<LAT, double> m;
+        if (fx_moments<LAT>([&](int i) { return g[i]; }, G.rho0, G.ref, stored_ref<S>(G, 0), stored_ref<S>(G, 1), m)) {
+            U[0] = m.s0;
+            U[1] = m.ux;
+            U[2] = m.uy;
+            U[3] = m.dT;
+        } else {
+            macros_wide<LAT, S>(G, in, U);
+        }
     }
     const long long n = (long long)y * G.nx + x;
     rho[n] = G.rho0 + U[0];

@@ -1,0 +1,351 @@
+// fix64.cuh -- FP64 sums and the FP64 collision on the integer pipe.
+//
+// One FP64 warp instruction takes 64 cycles of an SM sub-partition on GB300,
+// an integer one 1 to 2, so the FP64 update (467 FP64 instructions a D2Q37
+// node) was bound by that pipe at a tenth of the memory bandwidth.  Here the
+// additions and the products with the velocities' small integer components
+// are done in block fixed point: the numbers of one node are written as
+// integers times a common power of two taken from the largest of them, added
+// exactly, and rounded once when they become doubles again.  FP64 is left for
+// what is a product of two fields: the macros, the 15 monomial coefficients
+// of the equilibrium and two operations per stored population (about 140
+// instructions a node; the pipe stays 78 % busy, the issue slots 30 %).
+//
+// D2Q37 1024x512, 20 steps with initial fields and read-out: 10.43 -> 4.07 ms
+// (the bulk update 461 -> 170 us).  Against extended precision (a vortex in a
+// stream, 30 steps, 0.8 for tau) the velocities are no further off than with
+// FP64 sums: D2Q37 u_x 1.4e-15 and 1.5e-15, u_y 1.2e-14 and 4.0e-15; D2Q17
+// 4.3e-16 and 2.3e-16, 1.0e-14 and 4.5e-15; D2Q9 2.1e-15 and 2.0e-15, 8.2e-15
+// and 5.0e-15.
+#pragma once
+#include "lbm_internal.cuh"
+
+namespace lbmgb {
+
+// Biased exponent of a double from its high word.
+__device__ __forceinline__ int fx_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// Block exponents the fixed-point forms take: no infinities, NaN or overflow
+// above, no denormal results below; everything else goes to the FP64 forms.
+__device__ __forceinline__ bool fx_range(int e) { return e >= 128 && e <= 1900; }
+
+// The leading bit of a number of the block's largest exponent: kFxTop for the
+// equilibrium's monomials (at most 180 of them in one value, counted with
+// their factors) and for the non-equilibrium moments (at most 152), kFxSum for
+// the sums of populations (at most 52, in sum g c), so that all stay below 2^63.
+constexpr int kFxTop = 54, kFxSum = 56;
+
+// v in units of 2^(emax - 1023 - T), rounded to nearest (truncation is a
+// drift that adds up over the steps); |v| < 2^(emax - 1022), emax >= 128.
+template <int T>
+__device__ __forceinline__ long long fx_of(double v, int emax)
+{
+    const int hi = __double2hiint(v);
+    const unsigned long long m =
+        ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << (T - 51);
+    const int d = emax - ((hi >> 20) & 0x7ff);
+    const long long a = (long long)(((m >> (d < 63 ? d : 63)) + 1) >> 1), s = hi >> 31;
+    return (a ^ s) - s;
+}
+
+// The same for T = kFxTop with 32 more bits below, truncated.
+__device__ __forceinline__ __int128 fx_wide_of(double v, int emax)
+{
+    const int hi = __double2hiint(v);
+    const unsigned long long m =
+        (unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v);
+    // m << (32 + kFxTop - 52 - d) as high and low words
+    const int d = emax - ((hi >> 20) & 0x7ff), n = d < 95 ? d : 95;
+    unsigned long long h = m >> (64 - 32 - (kFxTop - 52)), l = m << (32 + kFxTop - 52);
+    if (n >= 64) {
+        l = h >> (n - 64);
+        h = 0;
+    } else if (n > 0) {
+        l = l >> n | h << (64 - n);
+        h >>= n;
+    }
+    const __int128 a = (__int128)((unsigned __int128)h << 64 | l);
+    return hi < 0 ? -a : a;
+}
+
+// x units of 2^(emax - 1023 - T) as a double, rounded to nearest.
+template <int T>
+__device__ __forceinline__ double fx_double(long long x, int emax)
+{
+    const long long s = x >> 63;
+    unsigned long long a = (unsigned long long)((x ^ s) - s);
+    const int n = __clzll((long long)a);
+    a <<= (n & 63);
+    const unsigned long long m = (a >> 11) + ((a >> 10) & 1);       // 53 bits, the leading one included
+    const unsigned e = (unsigned)(emax + (63 - T) - 1 - n) << 20;
+    const unsigned h = (unsigned)(m >> 32) + e + ((unsigned)s & 0x80000000u);
+    return a ? __hiloint2double((int)h, (int)(unsigned)m) : 0.0;
+}
+
+// A positive double as a 53-bit integer times a power of two, m 2^e, and the
+// weights of a lattice's classes as such.
+struct FxConst {
+    long long m;
+    int e;
+};
+template <int LAT>
+struct FxWeights {
+    FxConst w[Lat<LAT>::NCLS];
+    constexpr FxWeights() : w()
+    {
+        for (int k = 0; k < Lat<LAT>::NCLS; ++k) {
+            double v = Lat<LAT>::wcls(k);
+            int e = 0;
+            for (; v < 4503599627370496.0; --e) v *= 2.0;      // 2^52
+            w[k].m = (long long)v;
+            w[k].e = e;
+        }
+    }
+};
+
+// w times x units of 2^(emax - 1023 - kFxTop) as a double: 64 leading bits of
+// the product, rounded to nearest.
+__device__ __forceinline__ double fx_scaled(long long x, FxConst w, int emax)
+{
+    const long long s = x >> 63;
+    unsigned long long a = (unsigned long long)((x ^ s) - s);
+    const int n = __clzll((long long)a);
+    a = __umul64hi(a << (n & 63), (unsigned long long)w.m << 11);       // in [2^62, 2^64)
+    const int k = a >> 63 ? 0 : 1;
+    a <<= k;
+    const unsigned long long m = (a >> 11) + ((a >> 10) & 1);           // 53 bits, the leading one included
+    const unsigned e = (unsigned)(emax + w.e + (116 - kFxTop) - 1 - n - k) << 20;
+    const unsigned h = (unsigned)(m >> 32) + e + ((unsigned)s & 0x80000000u);
+    return x ? __hiloint2double((int)h, (int)(unsigned)m) : 0.0;
+}
+
+// The block exponent of populations get(0..Q-1), or 0 if the fixed-point
+// forms do not take them.  Populations that are all zero count as any block.
+template <int LAT, typename Get>
+__device__ __forceinline__ int fx_block(Get&& get)
+{
+    int emax = 0;
+    unsigned any = 0;
+#pragma unroll
+    for (int i = 0; i < Lat<LAT>::Q; ++i) {
+        const double v = get(i);
+        const int hi = __double2hiint(v) & 0x7fffffff;
+        emax = hi > emax ? hi : emax;
+        any |= unsigned(hi) | unsigned(__double2loint(v));
+    }
+    emax >>= 20;
+    return any == 0 ? 1023 : fx_range(emax) ? emax : 0;
+}
+
+// The sums of Eq. macro: s0 = sum g, (sx, sy) = sum g c, se = sum g |c|^2.
+template <int LAT, typename Get>
+__device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double& sx, double& sy, double& se)
+{
+    using L = Lat<LAT>;
+    long long E[L::NCLS], X[4] = {0, 0, 0, 0}, Y[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < L::NCLS; ++k) E[k] = 0;
+    E[0] = fx_of<kFxSum>(get(0), emax);
+#pragma unroll
+    for (int i = 1; i < L::Q; i += 2) {
+        const int cx = L::cx(i), cy = L::cy(i);
+        const long long p = fx_of<kFxSum>(get(i), emax), m = fx_of<kFxSum>(get(i + 1), emax), o = p - m;
+        E[L::cls(i)] += p + m;
+        if (cx > 0) X[cx] += o;
+        if (cx < 0) X[-cx] -= o;
+        if (cy > 0) Y[cy] += o;
+        if (cy < 0) Y[-cy] -= o;
+    }
+    // the energy's factors (216 in all) beyond 64 bits, rounded to units of 4
+    long long a0 = 0;
+    __int128 ae = 2;
+#pragma unroll
+    for (int k = 0; k < L::NCLS; ++k) {
+        a0 += E[k];
+        if (L::THERMAL) ae += (__int128)L::c2cls(k) * E[k];
+    }
+    s0 = fx_double<kFxSum>(a0, emax);
+    sx = fx_double<kFxSum>(X[1] + 2 * X[2] + 3 * X[3], emax);
+    sy = fx_double<kFxSum>(Y[1] + 2 * Y[2] + 3 * Y[3], emax);
+    se = L::THERMAL ? fx_double<kFxSum - 2>((long long)(ae >> 2), emax) : 0.0;
+}
+
+// Moments (Eq. macro) of populations get(i); false if they are out of range.
+template <int LAT, typename Get>
+__device__ __forceinline__ bool fx_moments(Get&& get, double rho0, int ref, double Ux, double Uy,
+                                           Moments<LAT, double>& m)
+{
+    const int emax = fx_block<LAT>(get);
+    if (emax == 0) return false;
+    double s0, sx, sy, se;
+    fx_sums<LAT>(get, emax, s0, sx, sy, se);
+    m = moments_of_sums<LAT, double>(s0, sx, sy, se, rho0, ref, Ux, Uy);
+    return true;
+}
+
+// The equilibrium (see eq_poly) of moments m held against w rho0, in the
+// monomials of (c_x, c_y):
+//   g^eq_i / w_i = sum over a + b <= ORDER of m_ab c_x^a c_y^b,
+// one value at a time to put(i, w, x, e): g^eq_i = fx_scaled(x, w, e).  False, with nothing put, if
+// the coefficients are out of the fixed-point range.  (jx, jy): the momentum
+// rho u.  All velocities share the coefficients' rounding, which in a uniform
+// stream adds up over the steps, so the linear ones, which carry the
+// momentum, are formed in three parts: the product j / c_s^2, its rounding
+// error, and the small nonlinear rest (drift of u without it: 3e-17 u a step).
+template <int LAT, typename Put>
+__device__ __forceinline__ bool fx_equilibrium(const Moments<LAT, double>& m, double jx, double jy, Put&& put)
+{
+    using L = Lat<LAT>;
+    using W = __int128;
+    constexpr bool O3 = L::ORDER >= 3, O4 = L::ORDER >= 4;
+    constexpr double ics2 = 1.0 / L::CS2;
+    const double X = m.ux * ics2, Y = m.uy * ics2;
+    const EqPoly<double> e = eq_poly<LAT, double>(m.ux * X + m.uy * Y, m.dT);
+    // coefficients: with p = c_x X + c_y Y and q = |c|^2,
+    // s0 + rho [A0 + B0' q + C0' q^2 + (A2 + B2' q) p^2 + p^4 / 24] and
+    // rho [(A1 + B1' q) p + p^3 / 6]
+    constexpr int NM = O4 ? 15 : O3 ? 10 : 6;
+    double c[NM];
+    const double rX = jx * ics2, rY = jy * ics2, XX = X * X, XY = X * Y, YY = Y * Y;
+    const double lX = fma(jx, ics2, -rX), lY = fma(jy, ics2, -rY);
+    const double rA2 = m.rho * e.A2, rB0 = m.rho * (e.B0 * ics2);
+    c[0] = m.s0 + m.rho * e.A0;             // 1
+    c[1] = rX;                              // x
+    c[2] = rY;                              // y
+    c[3] = rB0 + rA2 * XX;                  // x^2
+    c[4] = rB0 + rA2 * YY;                  // y^2
+    c[5] = 2.0 * rA2 * XY;                  // x y
+    if constexpr (O3) {
+        const double B1 = e.B1 * ics2;
+        c[6] = rX * (B1 + (1.0 / 6.0) * XX);    // x^3
+        c[7] = rY * (B1 + (1.0 / 6.0) * YY);    // y^3
+        c[8] = rY * (B1 + 0.5 * XX);            // x^2 y
+        c[9] = rX * (B1 + 0.5 * YY);            // x y^2
+    }
+    if constexpr (O4) {
+        const double rB2 = m.rho * (e.B2 * ics2), rC0 = m.rho * (e.C0 * (ics2 * ics2)), r4 = m.rho * (1.0 / 24.0);
+        c[10] = rC0 + XX * (rB2 + r4 * XX);                                     // x^4
+        c[11] = rC0 + YY * (rB2 + r4 * YY);                                     // y^4
+        c[12] = 2.0 * rC0 + (rB2 * (XX + YY) + (6.0 * r4) * (XX * YY));         // x^2 y^2
+        c[13] = XY * (2.0 * rB2 + (4.0 * r4) * XX);                             // x^3 y
+        c[14] = XY * (2.0 * rB2 + (4.0 * r4) * YY);                             // x y^3
+    }
+    int ec = 0;
+#pragma unroll
+    for (int k = 0; k < NM; ++k) ec = max(ec, fx_exp(c[k]));
+    if (ec == 0) ec = 1023;                 // all zero
+    if (!fx_range(ec)) return false;
+    W v[NM];
+#pragma unroll
+    for (int k = 0; k < NM; ++k) v[k] = fx_wide_of(c[k], ec);
+    v[1] += fx_wide_of(lX, ec);
+    v[2] += fx_wide_of(lY, ec);
+    if constexpr (O3) {                 // (A1 - 1) of eq_poly
+        const double a1 = fma(-0.5, m.ux * X + m.uy * Y, -2.0 * m.dT);
+        const double nx = rX * a1, ny = rY * a1;
+        if (fx_exp(nx) > ec || fx_exp(ny) > ec) return false;
+        v[1] += fx_wide_of(nx, ec);
+        v[2] += fx_wide_of(ny, ec);
+    }
+    // the parts below are rounded to 64 bits by adding this and dropping 32
+    const W half = W(1) << 31;
+    v[0] += half;
+    // per axis: even x^2 + x^4 and odd x + x^3 parts at |c| = 0 .. 3
+    W fx[4], fy[4], gx[4], gy[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        fx[a] = W(a * a) * v[3];
+        fy[a] = W(a * a) * v[4];
+        gx[a] = W(a) * v[1] + (a ? half : 0);
+        gy[a] = W(a) * v[2] + (a ? half : 0);
+        if constexpr (O3) {
+            gx[a] += W(a * a * a) * v[6];
+            gy[a] += W(a * a * a) * v[7];
+        }
+        if constexpr (O4) {
+            fx[a] += W(a * a * a * a) * v[10];
+            fy[a] += W(a * a * a * a) * v[11];
+        }
+    }
+    constexpr FxWeights<LAT> wt{};
+    put(0, wt.w[0], (long long)(v[0] >> 32), ec);
+#pragma unroll
+    for (int i = 1; i < L::Q; i += 2) {
+        const int cx = L::cx(i), cy = L::cy(i), a = cx < 0 ? -cx : cx, b = cy < 0 ? -cy : cy;
+        W Ev = (v[0] + fx[a]) + fy[b], Ox = gx[a], Oy = gy[b], Xy = 0;
+        if (a && b) {
+            Xy = W(a * b) * v[5] + half;
+            if constexpr (O3) {
+                Ox += W(a * b * b) * v[9];
+                Oy += W(a * a * b) * v[8];
+            }
+            if constexpr (O4) {
+                Ev += W(a * a * b * b) * v[12];
+                Xy += W(a * a * a * b) * v[13] + W(a * b * b * b) * v[14];
+            }
+        }
+        const long long ev = (long long)(Ev >> 32), xy = (long long)(Xy >> 32), ox = (long long)(Ox >> 32),
+                        oy = (long long)(Oy >> 32);
+        const long long E = cx * cy < 0 ? ev - xy : ev + xy;
+        const long long O = (cx < 0 ? -ox : ox) + (cy < 0 ? -oy : oy);
+        put(i, wt.w[L::cls(i)], E + O, ec);
+        put(i + 1, wt.w[L::cls(i)], E - O, ec);
+    }
+    return true;
+}
+
+// BGK collision (Eq. bgk) of the populations get(i) of a node with moments m;
+// post-collision values go to put(i, value).  g^eq is rounded before g is taken
+// from it, so that a node at equilibrium stays there: with the residue of an
+// unrounded product, omega > 1 moves it by a unit in the last place each step.
+template <int LAT, typename Get, typename Put>
+__device__ __forceinline__ bool fx_relax(const Moments<LAT, double>& m, double om, Get&& get, Put&& put)
+{
+    return fx_equilibrium<LAT>(m, m.sx, m.sy, [&](int i, FxConst w, long long x, int e) {
+        const double g = get(i);
+        put(i, fma(om, fx_scaled(x, w, e) - g, g));
+    });
+}
+
+// neq_moments (collide.cuh) with its sums in fixed point; get(i) in range.
+// The third moments are sum g (|c|^2 - 5) c + (5 - 4 c_s^2) sum g c, the product
+// with the constant in 128 bits: the two parts all but cancel.
+template <int LAT, typename Get>
+__device__ __forceinline__ void fx_neq_sums(Get&& get, int emax, double& pxy, double& dxy, double& pxx, double& pyy,
+                                            double& rx, double& ry)
+{
+    using L = Lat<LAT>;
+    long long axy = 0, ad = 0, axx = 0, ayy = 0, ax = 0, ay = 0, jx = 0, jy = 0;
+#pragma unroll
+    for (int i = 1; i < L::Q; i += 2) {
+        const int cx = L::cx(i), cy = L::cy(i), c2 = cx * cx + cy * cy;
+        const long long p = fx_of<kFxTop>(get(i), emax), m = fx_of<kFxTop>(get(i + 1), emax), e = p + m, o = p - m;
+        axy += (long long)(cx * cy) * e;
+        if (L::THERMAL) {
+            ad += (long long)(cx * cx - cy * cy) * e;
+            ax += (long long)((c2 - 5) * cx) * o;
+            ay += (long long)((c2 - 5) * cy) * o;
+            jx += (long long)cx * o;
+            jy += (long long)cy * o;
+        } else {
+            axx += (long long)(cx * cx) * e;
+            ayy += (long long)(cy * cy) * e;
+        }
+    }
+    pxy = fx_double<kFxTop>(axy, emax);
+    if (L::THERMAL) {
+        dxy = fx_double<kFxTop>(ad, emax);
+        // sums below 100 units of 2^(kFxTop + 1), the constant below 2^58
+        constexpr long long K = (long long)((5.0 - 4.0 * L::CS2) * double(1LL << 56));
+        const __int128 half = (__int128)1 << 55;
+        rx = fx_double<kFxTop>(ax + (long long)(((__int128)jx * K + half) >> 56), emax);
+        ry = fx_double<kFxTop>(ay + (long long)(((__int128)jy * K + half) >> 56), emax);
+        pxx = pyy = 0.0;
+    } else {
+        pxx = fx_double<kFxTop>(axx, emax);
+        pyy = fx_double<kFxTop>(ayy, emax);
+        dxy = rx = ry = 0.0;
+    }
+}
+
+}  // namespace lbmgb
