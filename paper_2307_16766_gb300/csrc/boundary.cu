@@ -42,6 +42,31 @@ constexpr int kCluster = 4;
 // four SMs, CTA r forming component / wave r of every unknown and exchanging
 // through distributed shared memory (band_tile).
 
+// Stage field of a band tile: stage values Y of its unknowns and strip macros
+// S of the stage time.  A strip node's macros at t, t + 1/2 and t + 1 are
+// three tables, formed once when the strip is read: interpolated at every
+// access they took 9 operations a stencil point, 45 a stage (with FP64
+// storage 64 cycles each).
+template <typename R>
+struct CtxB {
+    const R* Y;
+    const R* S;
+};
+template <typename R>
+__device__ __forceinline__ void fetch_local(const CtxB<R>& X, int ref, int kind, R r, R* Lc)
+{
+    const R* p = ref >= 0 ? X.Y + 4 * ref : X.S + 4 * (-ref - 1);
+    R U[4];
+    if constexpr (sizeof(R) == 8) {
+        const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+        U[0] = a.x; U[1] = a.y; U[2] = b.x; U[3] = b.y;
+    } else {
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        U[0] = a.x; U[1] = a.y; U[2] = a.z; U[3] = a.w;
+    }
+    to_local(kind, r, U, Lc);
+}
+
 // Share c of the mesoscopic viscous vector (see vis_meso), in arithmetic
 // type R: V1 for c = 1, V2 for c = 2; V3 is split, its conductive part for
 // c = 0 and its viscous-heating part for c = 3 (V0 = 0).
@@ -84,7 +109,7 @@ __device__ R vis_meso_c(int c, const Geom& G, const R* SU, const R* SN, const UD
 // Share c of the "-FD" viscous vector (see vis_fd), split as vis_meso_c:
 // V3 = (c = 0 part) + (c = 3 part).
 template <bool TH, typename R>
-__device__ R vis_fd_c(int c, const Geom& G, const Band& B, const CtxT<R>& X0, const UDesc& D, int u,
+__device__ R vis_fd_c(int c, const Geom& G, const Band& B, const CtxB<R>& X0, const UDesc& D, int u,
                       R cs2)
 {
     if (!TH && (c == 0 || c == 3)) return R(0);
@@ -215,6 +240,34 @@ __device__ __forceinline__ FF ff_addf(FF x, float b)
     return ff_fast(s.h, s.l + x.l);
 }
 
+// One strip node with FP32 / FP16 storage: the macros of t + 1 (returned), the
+// post-collision populations (into fx, if not null) and, if neq, the
+// non-equilibrium moments of t + 1.  (Inlined: as a function it took the 256^2
+// pulse from 2.21 to 2.80 ms a pass.)
+template <int LAT, typename S, bool REF>
+__device__ __forceinline__ float4 strip_node(const Geom& G, const Offsets& O, const S* __restrict__ fin, int x, int y,
+                                          S* fx, bool neq, float* N1)
+{
+    using L = Lat<LAT>;
+    float g[L::Q];
+    pull_plain<LAT, S, float>(G, O, fin, x, y, g);
+    if (Store<S>::SCALED) {
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) g[i] *= float(L::w(i));
+    }
+    Moments<LAT, float> m;
+    if (fx) {
+        m = collide<LAT, float, REF>(G, g, [&](int i, float v) {
+            if (Store<S>::SCALED) v *= float(1.0 / L::w(i));
+            Store<S>::put(fx + i, v);
+        });
+    } else {
+        m = moments_G<LAT, float, REF>(G, g);
+    }
+    if (neq) neq_moments<LAT, float, float>(g, m, 1.0f - 0.5f * omega_of<float>(G), N1);
+    return make_float4(m.s0, m.ux, m.uy, m.dT);
+}
+
 // One tile of the boundary band with FP32 / FP16 storage, in one CTA: the
 // phases of band_tile below (strip nodes, the four RK4 stages of the tile's
 // unknowns in shared memory, the Dirichlet write), with one thread carrying
@@ -255,7 +308,8 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
     extern __shared__ __align__(16) unsigned char dyn_raw[];
     float* SUt = reinterpret_cast<float*>(dyn_raw);    // [max_nodes][4] macros of t
     float* SUt1 = SUt + 4 * B.max_nodes;               // [max_nodes][4] macros of t + 1
-    float* SNt = SUt1 + 4 * B.max_nodes;               // [max_nodes][5] moments of t
+    float* SUh = SUt1 + 4 * B.max_nodes;               // [max_nodes][4] macros of t + 1/2
+    float* SNt = SUh + 4 * B.max_nodes;                // [max_nodes][5] moments of t
     S* Fx = reinterpret_cast<S*>(SNt + 5 * B.max_nodes);   // [max_fx][Q]
     const int ns = B.max_nodes;
     const UDesc D = B.ld[(long long)tile * kTileUnknowns + l];
@@ -285,8 +339,9 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
             const int kn = k + kPull;
             if (kn < ns) N0 = snt[kn];      // the next node's descriptor beside this one's pull
             if (N.x < 0) continue;
+            float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (N.flags & kSNLoadT) {
-                const float4 u = *reinterpret_cast<const float4*>(gU + 4LL * N.tslot);
+                u = *reinterpret_cast<const float4*>(gU + 4LL * N.tslot);
                 *reinterpret_cast<float4*>(SUt + 4 * k) = u;
                 if (meso) {
 #pragma unroll
@@ -294,30 +349,17 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
                 }
             }
             if (!(N.flags & kSNPull)) continue;
-            C g[L::Q];
-            pull_plain<LAT, S, C>(G, O, fin, N.x, N.y, g);
-            if (Store<S>::SCALED) {
-#pragma unroll
-                for (int i = 0; i < L::Q; ++i) g[i] *= C(L::w(i));
-            }
-            Moments<LAT, C> m;
-            if (N.fx >= 0) {
-                S* fx = Fx + N.fx * L::Q;
-                m = collide<LAT, C, REF>(G, g, [&](int i, C v) {
-                    if (Store<S>::SCALED) v *= C(1.0 / L::w(i));
-                    Store<S>::put(fx + i, v);
-                });
-            } else {
-                m = moments_G<LAT, C, REF>(G, g);
-            }
-            const float4 u1 = make_float4(m.s0, m.ux, m.uy, m.dT);
+            float N1[5];
+            const float4 u1 = strip_node<LAT, S, REF>(G, O, fin, N.x, N.y, N.fx >= 0 ? Fx + N.fx * L::Q : nullptr,
+                                                      N.gslot >= 0 && (N.flags & kSNNeq), N1);
             *reinterpret_cast<float4*>(SUt1 + 4 * k) = u1;
+            *reinterpret_cast<float4*>(SUh + 4 * k) =
+                make_float4(0.5f * u.x + 0.5f * u1.x, 0.5f * u.y + 0.5f * u1.y, 0.5f * u.z + 0.5f * u1.z,
+                            0.5f * u.w + 0.5f * u1.w);
             if (N.gslot >= 0) {             // the strips of t + 1, for the next step
                 const long long slot = (long long)(par_t ^ 1) * E.nslots + N.gslot;
                 *reinterpret_cast<float4*>(static_cast<float*>(E.stripU) + slot * 4) = u1;
                 if (N.flags & kSNNeq) {     // a node of the mesoscopic stencil
-                    float N1[5];
-                    neq_moments<LAT, C, float>(g, m, 1.0f - 0.5f * omega_of<float>(G), N1);
                     float* q = static_cast<float*>(E.stripN) + slot * 5;
 #pragma unroll
                     for (int c = 0; c < 5; ++c) q[c] = N1[c];
@@ -338,9 +380,7 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
     // inputs, 1: the viscous vector, 2: the waves, 3: the right-hand side and
     // RK4 update, 4: the Dirichlet write, 5: none); 8: all of it
     const int part = dry ? warp - kPull / 32 : 8;
-    CtxT<float> X;
-    X.St = SUt;
-    X.St1 = SUt1;
+    CtxB<float> X;
     const float rho0r = rho0_of<float>(G), cs2r = float(L::CS2), kr = B.kR_f;
     const bool side = lev <= 4 && D.kind < 4, corner = lev <= 4 && !side;
     const int scheme = side ? B.scheme[D.kind] : SCH_LODI;
@@ -367,7 +407,7 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
 #pragma unroll 1
     for (int stage = 0; stage < (dry ? 1 : 4); ++stage) {
         X.Y = Ys[stage & 1];
-        X.frac = stage == 0 ? 0.0f : (stage == 3 ? 1.0f : 0.5f);
+        X.S = stage == 0 ? SUt : (stage == 3 ? SUt1 : SUh);
         if (lev <= 3 - stage) {
             const int kind = D.kind;
             float Ul[4] = {0, 0, 0, 0}, dUn[4] = {0, 0, 0, 0}, TT[4] = {0, 0, 0, 0};
@@ -577,7 +617,8 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     extern __shared__ __align__(16) unsigned char dyn_raw[];
     R* SUt = reinterpret_cast<R*>(dyn_raw);        // [max_nodes][4] macros of t
     R* SUt1 = SUt + 4 * B.max_nodes;               // [max_nodes][4] macros of t + 1
-    R* SNt = SUt1 + 4 * B.max_nodes;               // [max_nodes][5] moments of t
+    R* SUh = SUt1 + 4 * B.max_nodes;               // [max_nodes][4] macros of t + 1/2
+    R* SNt = SUh + 4 * B.max_nodes;                // [max_nodes][5] moments of t
     S* Fx = reinterpret_cast<S*>(SNt + 5 * B.max_nodes);   // [max_fx][Q], node k in CTA k % 4
     auto bcast = [&](auto* p, auto v) {
         cg::cluster_group cl = cg::this_cluster();
@@ -651,6 +692,11 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
     };
     auto pull_t1 = [&](int k, const StripNode& N) {
         C g[L::Q];
+        R U0[4] = {0, 0, 0, 0};         // the node's macros of t, for t + 1/2
+        if (N.flags & kSNLoadT) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) U0[c] = gU[4LL * N.tslot + c];
+        }
         pull_plain<LAT, S, C>(G, O, fin, N.x, N.y, g);
         // sums and collision on the integer pipe (fix64.cuh) where the numbers
         // are in its range
@@ -667,6 +713,10 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
         const R U1[4] = {R(m.s0), R(m.ux), R(m.uy), R(m.dT)};
 #pragma unroll
         for (int c = 0; c < 4; ++c) bcast(SUt1 + 4 * k + c, U1[c]);
+        if (N.flags & kSNLoadT) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) bcast(SUh + 4 * k + c, R(0.5) * U0[c] + R(0.5) * U1[c]);
+        }
         if (N.gslot >= 0) {             // the strips of t + 1, for the next step
             R* u = static_cast<R*>(E.stripU) + ((long long)(par_t ^ 1) * E.nslots + N.gslot) * 4;
 #pragma unroll
@@ -720,10 +770,8 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
 
     // 2. RK4, component grp of every unknown
     const int rank = grp;
-    CtxT<R> X;
+    CtxB<R> X;
     X.Y = Ys;
-    X.St = SUt;
-    X.St1 = SUt1;
     const R rho0r = rho0_of<R>(G), cs2r = R(L::CS2), kr = bconst<R>(B.kR, B.kR_f);
     const R kAr = bconst<R>(B.kA, B.kA_f), kBr = bconst<R>(B.kB, B.kB_f), ihcsr = bconst<R>(B.ihcs, B.ihcs_f),
             csr_ = bconst<R>(B.cs, B.cs_f);
@@ -740,7 +788,7 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
             expect_bytes(&xbar[stage & 1], unsigned(kCluster * sizeof(double)) * ncomp);
             expect_bytes(&xbar[2 + (stage & 1)], unsigned(kCluster * sizeof(R)) * ncomp);
         }
-        X.frac = stage == 0 ? R(0) : (stage == 3 ? R(1) : R(0.5));
+        X.S = stage == 0 ? SUt : (stage == 3 ? SUt1 : SUh);
         R Ul[4] = {0, 0, 0, 0}, dUn[4] = {0, 0, 0, 0};
         R d_ut = 0;
         // A: inputs of the system, type R: 1/rho, the transversal terms,
@@ -749,6 +797,10 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
         if (comp) {
             const int kind = D.kind;
             R A[4], Bv[4], Up[4], Um[4];
+            // the components of dU/dn that row `rank` of S reads
+            auto reads = [&](int m) {
+                return TH ? (rank == 1 ? m == 2 : m == 0 || m == 3 || (m == 1 && rank >= 2)) : (rank == 1 ? m == 2 : m < 2);
+            };
             fetch_local(X, l, kind, kr, Ul);
             if (corner) {
                 // LODI along the outward diagonal, one-sided difference of
@@ -757,7 +809,8 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
                 fetch_local(X, D.nb[1], kind, kr, Bv);
                 const R kC = bconst<R>(B.kC, B.kC_f);
 #pragma unroll
-                for (int m = 0; m < 4; ++m) dUn[m] = (R(3) * Ul[m] - R(4) * A[m] + Bv[m]) * kC;
+                for (int m = 0; m < 4; ++m)
+                    if (reads(m)) dUn[m] = (R(3) * Ul[m] - R(4) * A[m] + Bv[m]) * kC;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) Up[m] = Um[m] = R(0);
             } else {
@@ -765,12 +818,14 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
                     fetch_local(X, D.nb[1], kind, kr, A);
                     fetch_local(X, D.nb[2], kind, kr, Bv);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) dUn[m] = R(0.5) * (R(3) * Ul[m] - R(4) * A[m] + Bv[m]);
+                    for (int m = 0; m < 4; ++m)
+                        if (reads(m)) dUn[m] = R(0.5) * (R(3) * Ul[m] - R(4) * A[m] + Bv[m]);
                 } else {                 // Eq. FD-dx-center at inner layers
                     fetch_local(X, D.nb[0], kind, kr, A);
                     fetch_local(X, D.nb[1], kind, kr, Bv);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) dUn[m] = R(0.5) * (A[m] - Bv[m]);
+                    for (int m = 0; m < 4; ++m)
+                        if (reads(m)) dUn[m] = R(0.5) * (A[m] - Bv[m]);
                 }
                 fetch_local(X, D.nb[4], kind, kr, Up);
                 fetch_local(X, D.nb[5], kind, kr, Um);
@@ -986,8 +1041,8 @@ constexpr int band_threads() { return band_mono<S>() ? 4 * kTileThreads : kTileT
 
 template <int LAT, typename S, bool REF>
 __global__ void __launch_bounds__(band_threads<S>(), 1)
-    k_band(Geom G, Offsets O, Band B, Export E, const S* __restrict__ fin, S* __restrict__ f,
-           int par_t)
+    k_band(const __grid_constant__ Geom G, const __grid_constant__ Offsets O, const __grid_constant__ Band B,
+           const __grid_constant__ Export E, const S* __restrict__ fin, S* __restrict__ f, int par_t)
 {
     if constexpr (band_mono<S>()) {
         for (int t = blockIdx.x; t < B.n_tiles; t += gridDim.x) {
@@ -1037,7 +1092,7 @@ __global__ void k_zg(Geom G, Band B, S* __restrict__ f)
 template <int LAT, typename S>
 size_t band_smem(const Band& B)
 {
-    return (size_t)B.max_nodes * 13 * sizeof(typename StripReal<S>::T) +
+    return (size_t)B.max_nodes * 17 * sizeof(typename StripReal<S>::T) +
            (size_t)B.max_fx * Lat<LAT>::Q * sizeof(S);
 }
 
