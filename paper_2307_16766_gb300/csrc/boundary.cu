@@ -264,7 +264,7 @@ __device__ __forceinline__ float4 strip_node(const Geom& G, const Offsets& O, co
     } else {
         m = moments_G<LAT, float, REF>(G, g);
     }
-    if (neq) neq_moments<LAT, float, float>(g, m, 1.0f - 0.5f * omega_of<float>(G), N1);
+    if (neq) neq_moments<LAT, float, float, !(REF || Store<S>::SCALED)>(g, m, 1.0f - 0.5f * omega_of<float>(G), N1);
     return make_float4(m.s0, m.ux, m.uy, m.dT);
 }
 

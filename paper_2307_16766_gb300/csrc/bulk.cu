@@ -593,7 +593,13 @@ __global__ void __launch_bounds__(kBulkThreads) k_macros(Geom G, const S* __rest
     if (x >= G.nx) return;
     const S* in = f + (long long)y * G.nxp + x;
     double U[4] = {0.0, 0.0, 0.0, 0.0};
-    auto finite = [&]() { return isfinite(U[0]) && isfinite(U[1]) && isfinite(U[2]) && isfinite(U[3]); };
+    // by the exponent fields (a comparison of doubles takes the FP64 pipe)
+    auto finite = [&]() {
+        bool ok = true;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ok = ok && (__double2hiint(U[c]) & 0x7ff00000) != 0x7ff00000;
+        return ok;
+    };
     if constexpr (sizeof(typename Store<S>::C) == 4) {
         float h[L::Q];
 #pragma unroll

@@ -62,11 +62,13 @@ __device__ __forceinline__ Moments<LAT, C> moments_G(const Geom& G, const C* g)
 // third moment is that of (|c|^2 - 4 c_s^2) c, so that the rounding of rho, u
 // and theta does not enter at their size.  With a reference the closed forms
 // are differences from the reference's.
-// FP32 keeps the sums over g - g^eq: the closed form is faster where the band
-// kernel is all there is (256^2: 2.12 ms a pass, 2.20 with the sums) and
-// slower beside a large bulk (1024x512: 3.48, 3.34; 96 runs: 30.5, 29.8), and
-// the gradients of short runs feel its different rounding.
-// FP32 and derivative numbers: from the evaluated equilibrium.
+// FP32 and derivative numbers (EVAL) keep the sums over g - g^eq: the closed
+// form is faster where the band kernel is all there is (256^2: 2.12 ms a pass,
+// 2.20 with the sums) and slower beside a large bulk (1024x512: 3.48, 3.34; 96
+// runs: 30.5, 29.8), and the gradients of short runs feel its different
+// rounding.  FP16 storage and populations relative to a reference, where
+// there are no gradients, take the closed form: 4096^2 FP16 10.6 ms a pass
+// (11.6 with the sums), 1024x512 with a reference 3.8 (4.0).
 template <int LAT, typename C, typename T>
 __device__ __forceinline__ void neq_evaluated(const C* g, const Moments<LAT, C>& m, T fac, T* N)
 {
@@ -104,12 +106,12 @@ __device__ __forceinline__ void neq_evaluated(const C* g, const Moments<LAT, C>&
 template <int LAT, typename C, typename T>
 __device__ __forceinline__ void neq_close(const Moments<LAT, C>& m, T fac, T* N, C pxy, C dxy, C pxx, C pyy, C rx, C ry);
 
-template <int LAT, typename C, typename T>
+template <int LAT, typename C, typename T, bool EVAL = !std::is_same_v<C, double>>
 __device__ __forceinline__ void neq_moments(const C* g, const Moments<LAT, C>& m, T fac, T* N)
 {
     using L = Lat<LAT>;
     constexpr double cs2 = L::CS2;
-    if constexpr (!std::is_same_v<C, double>) return neq_evaluated<LAT, C, T>(g, m, fac, N);
+    if constexpr (EVAL) return neq_evaluated<LAT, C, T>(g, m, fac, N);
     // sum g c_x c_y; sum g (c_x^2 - c_y^2) per class (thermal) or sum g c_a^2
     // (D2Q9); sum g (|c|^2 - 4 c_s^2) c_a
     C pxy = 0, dxy = 0, pxx = 0, pyy = 0, rx = 0, ry = 0;
