@@ -785,7 +785,7 @@ int bulk(lbm_handle* h, int par, cudaStream_t st, int chain = CHAIN_NONE)
     int rc = mark(h, 0, st);
     if (rc != LBM_OK) return rc;
     rc = launch_bulk(h->lattice, h->storage, h->G, h->O, h->bulk, h->tmap[par], h->f[par],
-                     h->f[par ^ 1], h->flag + 1, st, chain);
+                     h->f[par ^ 1], h->flag + 1, st, chain, h->B.n_tiles == 0);
     if (rc) return check_launch(h, rc, "bulk kernel");
     return mark(h, 1, st);
 }
@@ -1042,7 +1042,7 @@ int lbm_step(lbm_handle* h, int n)
             // no characteristic side: bulk, inflow and zero gradient in order
             // (no early start after an inflow kernel)
             if (h->n_inflow > 0 && !(h->inflow_done[0] && h->inflow_done[1])) early = false;
-            rc = bulk(h, par, h->stream, early ? CHAIN_BULK : CHAIN_NONE);
+            rc = bulk(h, par, h->stream, early && !h->G.ref ? CHAIN_BULK : CHAIN_NONE);
             if (rc == LBM_OK) rc = band(h, par, h->stream);
             if (rc == LBM_OK) rc = zero_gradient(h, par, h->stream);
             if (rc != LBM_OK) return rc;

@@ -1110,7 +1110,7 @@ int boundary_t(const Geom& G, const Offsets& O, const Export& E, const Band& B, 
     // waits for (band, bulk, then this kernel) takes longer than a launch
     // when the band kernel is short: FP32 256^2 20.6 us a step without,
     // 22.2 us with; 1024x512 34.2, 38.9.
-    early = early && !mono;
+    early = early && !mono && !G.ref;   // (k_bulk_ref does not carry the chain)
     constexpr int ncl = mono ? 1 : kCluster;
     const dim3 grd(mono ? std::max(1, std::min(B.grid, B.n_tiles)) : B.n_tiles * ncl), blk(band_threads<S>());
     if (G.ref)

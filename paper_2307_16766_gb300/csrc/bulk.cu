@@ -281,26 +281,32 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
     }
 }
 
-// The next step's first kernel may be launched once every CTA of this grid
-// has begun (it waits for this grid's completion): periodic D2Q37 2048x1024
-// FP32 106.6 us a step without, 104.5 us with.  Beside a band kernel
-// (CHAIN_BAND) the last CTA stays until that kernel is complete, so that this
-// grid's completion stands for the whole step's.
-__device__ __forceinline__ void bulk_end(int chain)
+template <int LAT, typename S>
+__global__ void __launch_bounds__(kBulkThreads)
+    k_bulk(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
+           S* __restrict__ fout, int* status)
 {
-    if (chain == CHAIN_BAND && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && threadIdx.x == 0)
-        pdl_wait();
+    bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status, CHAIN_NONE);
 }
 
-// (FP64: three CTAs per SM, all that 168 registers of D2Q37 leave room for.)
+// The form of a step whose successor starts early (FP64 storage, and steps
+// without characteristic sides).  The next step's first kernel may be launched
+// once every CTA of this grid has begun (it waits for this grid's completion):
+// periodic D2Q37 2048x1024 FP32 106.6 us a step without, 104.5 us with.  Beside
+// a band kernel (CHAIN_BAND) the last CTA stays until that kernel is complete,
+// so that this grid's completion stands for the whole step's.  A kernel of its
+// own: with these lines in k_bulk, FP16 on 4096^2 took 11.42 ms a pass, 11.14
+// without.  (FP64: three CTAs per SM, all that 168 registers of D2Q37 leave
+// room for.)
 template <int LAT, typename S>
 __global__ void __launch_bounds__(kBulkThreads, sizeof(S) == 8 ? 3 : 0)
-    k_bulk(const __grid_constant__ Maps tm, const __grid_constant__ Geom G, const __grid_constant__ Offsets O, Region R,
-           const S* __restrict__ fin, S* __restrict__ fout, int* status, int chain)
+    k_bulk_chain(const __grid_constant__ Maps tm, const __grid_constant__ Geom G, const __grid_constant__ Offsets O,
+                 Region R, const S* __restrict__ fin, S* __restrict__ fout, int* status, int chain)
 {
     pdl_trigger();
     bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status, chain);
-    bulk_end(chain);
+    if (chain == CHAIN_BAND && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && threadIdx.x == 0)
+        pdl_wait();
 }
 
 // With a reference equilibrium: about twice the equilibrium arithmetic per
@@ -309,11 +315,9 @@ __global__ void __launch_bounds__(kBulkThreads, sizeof(S) == 8 ? 3 : 0)
 template <int LAT, typename S>
 __global__ void __launch_bounds__(kBulkThreads)
     k_bulk_ref(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
-               S* __restrict__ fout, int* status, int chain)
+               S* __restrict__ fout, int* status)
 {
-    pdl_trigger();
-    bulk_body<LAT, S, true>(tm, G, O, R, fin, fout, status, chain);
-    bulk_end(chain);
+    bulk_body<LAT, S, true>(tm, G, O, R, fin, fout, status, CHAIN_NONE);
 }
 
 // Persistent form of k_bulk for one or many grids of one lattice and
@@ -650,7 +654,7 @@ int inflow_t(const Geom& G, const int* nodes, int n, const double U[4], void* f,
 
 template <int LAT, typename S>
 int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* tmaps,
-           const void* fin, void* fout, int* status, cudaStream_t st, int chain)
+           const void* fin, void* fout, int* status, cudaStream_t st, int chain, bool follow)
 {
     const int h = R.y1 - R.y0;
     if (R.x1 <= R.x0 || h <= 0) return 0;
@@ -662,19 +666,22 @@ int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* 
     tm.m2 = tmaps[3];
     tm.m1 = tmaps[4];
     const dim3 blk(kBulkThreads);
-    const bool early = chain != CHAIN_NONE;
     if (G.ref) {
         constexpr int ROWS = bulk_rows<S, true>();
         constexpr size_t smem = ROWS * Stage<LAT, S>::TOTAL;
         static_assert(smem <= 48 * 1024, "bulk staging above the default dynamic shared memory");
-        return launch_ex(k_bulk_ref<LAT, S>, dim3(t1 - t0, (h + ROWS - 1) / ROWS), blk, smem, st, early, tm, G, O,
-                         R, static_cast<const S*>(fin), static_cast<S*>(fout), status, chain);
+        return launch_ex(k_bulk_ref<LAT, S>, dim3(t1 - t0, (h + ROWS - 1) / ROWS), blk, smem, st,
+                         chain == CHAIN_BAND, tm, G, O, R, static_cast<const S*>(fin), static_cast<S*>(fout), status);
     }
     constexpr int ROWS = bulk_rows<S, false>();
     constexpr size_t smem = ROWS * Stage<LAT, S>::TOTAL;
     static_assert(smem <= 48 * 1024, "bulk staging above the default dynamic shared memory");
-    return launch_ex(k_bulk<LAT, S>, dim3(t1 - t0, (h + ROWS - 1) / ROWS), blk, smem, st, early, tm, G, O, R,
-                     static_cast<const S*>(fin), static_cast<S*>(fout), status, chain);
+    const dim3 grd(t1 - t0, (h + ROWS - 1) / ROWS);
+    if (sizeof(S) == 8 || follow)
+        return launch_ex(k_bulk_chain<LAT, S>, grd, blk, smem, st, chain != CHAIN_NONE, tm, G, O, R,
+                         static_cast<const S*>(fin), static_cast<S*>(fout), status, chain);
+    return launch_ex(k_bulk<LAT, S>, grd, blk, smem, st, chain == CHAIN_BAND, tm, G, O, R,
+                     static_cast<const S*>(fin), static_cast<S*>(fout), status);
 }
 
 template <int LAT, typename S>
@@ -742,9 +749,9 @@ int launch_inflow(int lat, int storage, const Geom& G, const int* nodes, int n, 
 
 int launch_bulk(int lat, int storage, const Geom& G, const Offsets& O, const Region& R,
                 const CUtensorMap* tmaps, const void* fin, void* fout, int* status,
-                cudaStream_t st, int chain)
+                cudaStream_t st, int chain, bool follow)
 {
-#define CALL(L, S) bulk_t<L, S>(G, O, R, tmaps, fin, fout, status, st, chain)
+#define CALL(L, S) bulk_t<L, S>(G, O, R, tmaps, fin, fout, status, st, chain, follow)
     LBM_DISPATCH(lat, storage, CALL);
 #undef CALL
 }

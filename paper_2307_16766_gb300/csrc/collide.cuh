@@ -67,8 +67,8 @@ __device__ __forceinline__ Moments<LAT, C> moments_G(const Geom& G, const C* g)
 // 2.20 with the sums) and slower beside a large bulk (1024x512: 3.48, 3.34; 96
 // runs: 30.5, 29.8), and the gradients of short runs feel its different
 // rounding.  FP16 storage and populations relative to a reference, where
-// there are no gradients, take the closed form: 4096^2 FP16 10.6 ms a pass
-// (11.6 with the sums), 1024x512 with a reference 3.8 (4.0).
+// there are no gradients, take the closed form: 1024x512 with a reference 3.87 ms
+// a pass (4.00 with the sums), 4096^2 FP16 11.59 (11.65).
 template <int LAT, typename C, typename T>
 __device__ __forceinline__ void neq_evaluated(const C* g, const Moments<LAT, C>& m, T fac, T* N)
 {

@@ -810,10 +810,11 @@ int launch_inflow(int lat, int storage, const Geom& G, const int* nodes, int n, 
 // if a copy never completed.  chain: CHAIN_NONE (ordinary launch),
 // CHAIN_BAND (starts early beside the band kernel of the same step, whose
 // CTAs signal after the previous step is complete) or CHAIN_BULK (starts early
-// after the previous step's bulk kernel and waits for it).
+// after the previous step's bulk kernel and waits for it; not with a
+// reference).  follow: the next launch may be a CHAIN_BULK one.
 int launch_bulk(int lat, int storage, const Geom& G, const Offsets& O, const Region& R,
                 const CUtensorMap* tmaps, const void* fin, void* fout, int* status,
-                cudaStream_t st, int chain = CHAIN_NONE);
+                cudaStream_t st, int chain = CHAIN_NONE, bool follow = false);
 int launch_macros(int lat, int storage, const Geom& G, const void* f, double* rho, double* ux,
                   double* uy, double* T, int* flag, cudaStream_t st);
 // The band of one step fin -> fnew: strip nodes, RK4 of the characteristic
