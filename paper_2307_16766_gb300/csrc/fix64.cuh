@@ -8,7 +8,7 @@
 // integers times a common power of two taken from the largest of them, added
 // exactly, and rounded once when they become doubles again.  FP64 is left for
 // what is a product of two fields: the macros, the 15 monomial coefficients
-// of the equilibrium and two operations per stored population (about 140
+// of the equilibrium and two operations per stored population (154
 // instructions a node; the pipe stays 78 % busy, the issue slots 30 %).
 //
 // D2Q37 1024x512, 20 steps with initial fields and read-out: 10.43 -> 4.07 ms
