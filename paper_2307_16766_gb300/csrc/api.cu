@@ -41,7 +41,7 @@ struct lbm_handle {
     bool inflow_done[2] = {false, false};   // buffer already holds the inflow equilibrium
     double Uin[4] = {0, 0, 0, 0};
     double* macro = nullptr;
-    int* flag = nullptr;     // [0]: non-finite macros seen, [1]: kernel status bits
+    int* flag = nullptr;     // [0]: non-finite macros seen, [1]: kernel status bits, [2]: announce_step
     CUtensorMap tmap[2][5];  // tensor-copy descriptors of the two buffers, box depths 7, 5, 3, 2, 1
     void* ws = nullptr;
     size_t ws_bytes = 0;
@@ -597,7 +597,7 @@ int make_plan(int lattice, int nx, int ny, double tau, const lbm_cbc_params* p, 
     pl.off_zg = take(pl.zg.size() * sizeof(int2));
     pl.off_in = take(pl.inflow.size() * sizeof(int));
     pl.off_macro = take((size_t)4 * nx * ny * 8);
-    pl.off_flag = take(2 * sizeof(int));
+    pl.off_flag = take(3 * sizeof(int));
     pl.total = o;
     return LBM_OK;
 }
@@ -748,7 +748,7 @@ int setup(lbm_handle* h, int lattice, int nx, int ny, double tau, const lbm_cbc_
     e = cudaMemsetAsync(h->f[0], 0, h->f_bytes, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->f[1], 0, h->f_bytes, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->E.stripU, 0, pl.stripU_n * h->E.sesize, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flag, 0, 2 * sizeof(int), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->flag, 0, 3 * sizeof(int), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->E.stripN, 0, pl.stripN_n * h->E.sesize, h->stream);
     if (e == cudaSuccess && !pl.ud.empty())
         e = cudaMemcpyAsync(const_cast<UDesc*>(h->B.ud), pl.ud.data(), pl.ud.size() * sizeof(UDesc),
@@ -785,7 +785,7 @@ int bulk(lbm_handle* h, int par, cudaStream_t st, int chain = CHAIN_NONE)
     int rc = mark(h, 0, st);
     if (rc != LBM_OK) return rc;
     rc = launch_bulk(h->lattice, h->storage, h->G, h->O, h->bulk, h->tmap[par], h->f[par],
-                     h->f[par ^ 1], h->flag + 1, st, chain, h->B.n_tiles == 0);
+                     h->f[par ^ 1], par, h->flag + 1, st, chain, h->B.n_tiles == 0);
     if (rc) return check_launch(h, rc, "bulk kernel");
     return mark(h, 1, st);
 }
@@ -979,7 +979,7 @@ int lbm_init_fields(lbm_handle* h, const double* rho, const double* ux, const do
     int rc = launch_init(h->lattice, h->storage, h->G, h->E, h->B, dr, du, dv, dt, h->f[0], h->stream);
     if (rc) return check_launch(h, rc, "init kernels");
     h->inflow_done[0] = h->inflow_done[1] = false;
-    cudaError_t e = cudaMemsetAsync(h->flag, 0, 2 * sizeof(int), h->stream);   // a fresh state, no status
+    cudaError_t e = cudaMemsetAsync(h->flag, 0, 3 * sizeof(int), h->stream);   // a fresh state, no status
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "init");
     h->steps = 0;

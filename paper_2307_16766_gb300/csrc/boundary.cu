@@ -596,7 +596,7 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
 //    (equilibrium or Eq. NEEP), shared out over the four groups.
 template <int LAT, typename S, bool REF, bool BATCH>
 __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const Band& B,
-                                          const Export& E, const S* __restrict__ fin,
+                                          const Export& E, const S* fin,
                                           S* __restrict__ f, int par_t, int tile)
 {
     using L = Lat<LAT>;
@@ -673,6 +673,7 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
         // bulk update.  Once that step is complete, the bulk update of this
         // one (which reads only the old buffer) may begin.
         pdl_wait();
+        if (tile == 0 && grp == 0 && l == 0) announce_step(B.status, par_t);
         pdl_trigger();
     }
 
@@ -697,7 +698,7 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
 #pragma unroll
             for (int c = 0; c < 4; ++c) U0[c] = gU[4LL * N.tslot + c];
         }
-        pull_plain<LAT, S, C>(G, O, fin, N.x, N.y, g);
+        pull_plain<LAT, S, C, !BATCH>(G, O, fin, N.x, N.y, g);
         // sums and collision on the integer pipe (fix64.cuh) where the numbers
         // are in its range
         Moments<LAT, C> m;
@@ -1042,7 +1043,7 @@ constexpr int band_threads() { return band_mono<S>() ? 4 * kTileThreads : kTileT
 template <int LAT, typename S, bool REF>
 __global__ void __launch_bounds__(band_threads<S>(), 1)
     k_band(const __grid_constant__ Geom G, const __grid_constant__ Offsets O, const __grid_constant__ Band B,
-           const __grid_constant__ Export E, const S* __restrict__ fin, S* __restrict__ f, int par_t)
+           const __grid_constant__ Export E, const S* fin, S* __restrict__ f, int par_t)
 {
     if constexpr (band_mono<S>()) {
         for (int t = blockIdx.x; t < B.n_tiles; t += gridDim.x) {

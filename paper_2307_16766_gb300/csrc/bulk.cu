@@ -208,9 +208,12 @@ __device__ __forceinline__ void collide_store(const Geom& G, const Offsets& O, S
 template <typename S, bool REF>
 constexpr int bulk_rows() { return (sizeof(S) <= 4 && !REF) ? 2 : 1; }
 
-template <int LAT, typename S, bool REF>
+// EARLY: the launch may start before the previous step is complete (chain
+// says what it waits for then; par: parity of the step).
+template <int LAT, typename S, bool REF, bool EARLY = false>
 __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const Offsets& O, const Region& R,
-                                          const S* __restrict__ fin, S* __restrict__ fout, int* status, int chain)
+                                          const S* fin, S* __restrict__ fout, int* status, int chain = CHAIN_NONE,
+                                          int par = 0)
 {
     constexpr int ROWS = bulk_rows<S, REF>();
     using L = Lat<LAT>;
@@ -237,7 +240,10 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[r])));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (chain == CHAIN_BULK) pdl_wait();
+        if constexpr (EARLY) {
+            if (chain == CHAIN_BULK) pdl_wait();
+            if (sizeof(S) == 8 && chain == CHAIN_BAND) await_step(status, par);
+        }
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             if (!staged(yb + r)) continue;
@@ -248,7 +254,7 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
                                  std::make_integer_sequence<int, L::NG>{});
         }
     }
-    if (chain == CHAIN_BULK) pdl_wait();
+    if (EARLY && chain == CHAIN_BULK) pdl_wait();
     __syncthreads();
 #pragma unroll 1
     for (int r = 0; r < ROWS; ++r) {
@@ -270,7 +276,7 @@ __device__ __forceinline__ void bulk_body(const Maps& tm, const Geom& G, const O
                                          std::make_integer_sequence<int, Q>{});
         } else {
             if (!valid) continue;
-            pull_plain<LAT, S, C>(G, O, fin, x, y, g);
+            pull_plain<LAT, S, C, EARLY>(G, O, fin, x, y, g);
             if constexpr (FIXED)
                 put_staged<LAT, S>(g, reinterpret_cast<S*>(smem_raw + r * BX::TOTAL) + threadIdx.x);
         }
@@ -286,7 +292,7 @@ __global__ void __launch_bounds__(kBulkThreads)
     k_bulk(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
            S* __restrict__ fout, int* status)
 {
-    bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status, CHAIN_NONE);
+    bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status);
 }
 
 // The form of a step whose successor starts early (FP64 storage, and steps
@@ -301,10 +307,10 @@ __global__ void __launch_bounds__(kBulkThreads)
 template <int LAT, typename S>
 __global__ void __launch_bounds__(kBulkThreads, sizeof(S) == 8 ? 3 : 0)
     k_bulk_chain(const __grid_constant__ Maps tm, const __grid_constant__ Geom G, const __grid_constant__ Offsets O,
-                 Region R, const S* __restrict__ fin, S* __restrict__ fout, int* status, int chain)
+                 Region R, const S* fin, S* __restrict__ fout, int* status, int chain, int par)
 {
     pdl_trigger();
-    bulk_body<LAT, S, false>(tm, G, O, R, fin, fout, status, chain);
+    bulk_body<LAT, S, false, true>(tm, G, O, R, fin, fout, status, chain, par);
     if (chain == CHAIN_BAND && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && threadIdx.x == 0)
         pdl_wait();
 }
@@ -317,7 +323,7 @@ __global__ void __launch_bounds__(kBulkThreads)
     k_bulk_ref(const __grid_constant__ Maps tm, Geom G, Offsets O, Region R, const S* __restrict__ fin,
                S* __restrict__ fout, int* status)
 {
-    bulk_body<LAT, S, true>(tm, G, O, R, fin, fout, status, CHAIN_NONE);
+    bulk_body<LAT, S, true>(tm, G, O, R, fin, fout, status);
 }
 
 // Persistent form of k_bulk for one or many grids of one lattice and
@@ -654,7 +660,7 @@ int inflow_t(const Geom& G, const int* nodes, int n, const double U[4], void* f,
 
 template <int LAT, typename S>
 int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* tmaps,
-           const void* fin, void* fout, int* status, cudaStream_t st, int chain, bool follow)
+           const void* fin, void* fout, int par, int* status, cudaStream_t st, int chain, bool follow)
 {
     const int h = R.y1 - R.y0;
     if (R.x1 <= R.x0 || h <= 0) return 0;
@@ -679,7 +685,7 @@ int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* 
     const dim3 grd(t1 - t0, (h + ROWS - 1) / ROWS);
     if (sizeof(S) == 8 || follow)
         return launch_ex(k_bulk_chain<LAT, S>, grd, blk, smem, st, chain != CHAIN_NONE, tm, G, O, R,
-                         static_cast<const S*>(fin), static_cast<S*>(fout), status, chain);
+                         static_cast<const S*>(fin), static_cast<S*>(fout), status, chain, par);
     return launch_ex(k_bulk<LAT, S>, grd, blk, smem, st, chain == CHAIN_BAND, tm, G, O, R,
                      static_cast<const S*>(fin), static_cast<S*>(fout), status);
 }
@@ -748,10 +754,10 @@ int launch_inflow(int lat, int storage, const Geom& G, const int* nodes, int n, 
 }
 
 int launch_bulk(int lat, int storage, const Geom& G, const Offsets& O, const Region& R,
-                const CUtensorMap* tmaps, const void* fin, void* fout, int* status,
+                const CUtensorMap* tmaps, const void* fin, void* fout, int par, int* status,
                 cudaStream_t st, int chain, bool follow)
 {
-#define CALL(L, S) bulk_t<L, S>(G, O, R, tmaps, fin, fout, status, st, chain, follow)
+#define CALL(L, S) bulk_t<L, S>(G, O, R, tmaps, fin, fout, par, status, st, chain, follow)
     LBM_DISPATCH(lat, storage, CALL);
 #undef CALL
 }

@@ -191,10 +191,13 @@ __device__ __forceinline__ void neq_close(const Moments<LAT, C>& m, T fac, T* N,
     }
 }
 
-// Plain pull of node (x, y) with periodic wrap-around of the sources.
-template <int LAT, typename S, typename C>
-__device__ __forceinline__ void pull_plain(const Geom& G, const Offsets& O,
-                                           const S* __restrict__ fin, int x, int y, C* g)
+// Plain pull of node (x, y) with periodic wrap-around of the sources.  LIVE:
+// the previous step may still have been writing fin when this kernel started
+// (early start), so the loads are ordinary ones, which the wait for that step
+// orders; fin must not come from a const __restrict__ kernel parameter then,
+// which would make them read-only loads again.
+template <int LAT, typename S, typename C, bool LIVE = false>
+__device__ __forceinline__ void pull_plain(const Geom& G, const Offsets& O, const S* fin, int x, int y, C* g)
 {
     using L = Lat<LAT>;
 #pragma unroll
@@ -202,7 +205,9 @@ __device__ __forceinline__ void pull_plain(const Geom& G, const Offsets& O,
         int xs = x - L::cx(i), ys = y - L::cy(i);
         if (L::cx(i) && G.perx) xs = xs < 0 ? xs + G.nx : (xs >= G.nx ? xs - G.nx : xs);
         if (L::cy(i) && G.pery) ys = ys < 0 ? ys + G.ny : (ys >= G.ny ? ys - G.ny : ys);
-        g[i] = C(Store<S>::load(fin + (O.st[i] + ys * G.nxp + xs)));
+        const S* p = fin + (O.st[i] + ys * G.nxp + xs);
+        if constexpr (LIVE) g[i] = C(Store<S>::value(*p));
+        else g[i] = C(Store<S>::load(p));
     }
 }
 
