@@ -445,6 +445,11 @@ __global__ void __launch_bounds__(kBulkThreads)
                                     reinterpret_cast<double*>(out), nullptr, plane);
             else collide<LAT, C, false>(R.G, g, put);
         }
+        // plain stores of put_staged before the tensor copies that refill the
+        // buffer: a CTA barrier alone orders them for other threads' plain
+        // accesses, not for the copies' (asynchronous) proxy
+        if constexpr (bulk_fixed<S, false>())
+            if (!cur.staged) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();                    // stage buffer read by all before its reuse
         w = wn;
         cur = nxt;
