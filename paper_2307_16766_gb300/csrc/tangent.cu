@@ -287,9 +287,10 @@ __global__ void k_tl_stage(Geom G, Band B, Relax<TB<S>> P, const TB<S>* __restri
 // unknown's band node (corner: its M x M block), value and derivatives, in
 // the storage's arithmetic.  Thread (u, k) takes derivative direction k of
 // unknown u on Dual<., 1> numbers (direction 0 also writes the values):
-// three short chains per unknown instead of one long one.
+// three short chains per unknown instead of one long one.  (Uf is still being
+// written when this kernel starts: no read-only loads, so no __restrict__.)
 template <int LAT, typename S>
-__global__ void k_tl_dirichlet(Geom G, Band B, const TB<S>* __restrict__ Uf, S* __restrict__ f,
+__global__ void k_tl_dirichlet(Geom G, Band B, const TB<S>* Uf, S* __restrict__ f,
                                S* __restrict__ t)
 {
     using L = Lat<LAT>;
