@@ -501,9 +501,12 @@ __global__ void k_init(Geom G, Export E, const double* __restrict__ rho,
     S* out = f + (long long)y * G.nxp + x;
     bool done = false;
     if constexpr (sizeof(S) == 8)       // FP64 on the integer pipe, as the bulk update
-        if (!G.ref) done = fx_equilibrium<LAT>(mc, mc.rho * mc.ux, mc.rho * mc.uy, [&](int i, FxConst w, long long x, int e) {
+        if (!G.ref) {
+            const double se = 2.0 * L::CS2 * mc.s0 + mc.rho * (mc.ux * mc.ux + mc.uy * mc.uy + 2.0 * L::CS2 * mc.dT);
+            done = fx_equilibrium<LAT>(mc, mc.rho * mc.ux, mc.rho * mc.uy, se, [&](int i, FxConst w, long long x, int e) {
                 out[L::plane_of(i) * G.plane] = fx_scaled(x, w, e);
             });
+        }
     if (!done) {
         C geq[L::Q];
         equilibrium<LAT, C>(mc, geq);

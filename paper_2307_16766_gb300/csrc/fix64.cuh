@@ -7,16 +7,18 @@
 // are done in block fixed point: the numbers of one node are written as
 // integers times a common power of two taken from the largest of them, added
 // exactly, and rounded once when they become doubles again.  FP64 is left for
-// what is a product of two fields: the macros, the 15 monomial coefficients
-// of the equilibrium and two operations per stored population (154
-// instructions a node; the pipe stays 78 % busy, the issue slots 30 %).
+// what is a product of two fields: the macros, the monomial coefficients of
+// the equilibrium and two operations per stored population (142 instructions a
+// D2Q37 node: 140 of the 174 us of an update of 1024x512, the rest waits on it).
 //
-// D2Q37 1024x512, 20 steps with initial fields and read-out: 10.43 -> 4.07 ms
-// (the bulk update 461 -> 170 us).  Against extended precision (a vortex in a
-// stream, 30 steps, 0.8 for tau) the velocities are no further off than with
-// FP64 sums: D2Q37 u_x 1.4e-15 and 1.5e-15, u_y 1.2e-14 and 4.0e-15; D2Q17
-// 4.3e-16 and 2.3e-16, 1.0e-14 and 4.5e-15; D2Q9 2.1e-15 and 2.0e-15, 8.2e-15
-// and 5.0e-15.
+// D2Q37 1024x512, 20 steps with initial fields and read-out: 10.43 -> 3.96 ms
+// (the bulk update 461 -> 174 us).  Errors of the velocities against extended
+// precision (80 bits), geometric mean over 8 to 16 flows of 20 to 80 steps,
+// tau 0.55 to 1.1, beside those of FP64 sums and an FP64 equilibrium:
+//   a stream, periodic   D2Q9 1.1e-17, 1.4e-17; D2Q17 1.2e-17, 3.8e-17; D2Q37 9.1e-18, 1.1e-16
+//   ... through CBC sides D2Q9 1.3e-17, 2.0e-17; D2Q17 1.1e-17, 2.6e-17; D2Q37 9.3e-18, 3.8e-17
+//   from rest            D2Q9 1.7e-19, 2.4e-19; D2Q17 9.5e-20, 2.4e-19; D2Q37 3.4e-20, 3.2e-19
+// (u_x; u_y, density and temperature are no further off in any row either).
 #pragma once
 #include "lbm_internal.cuh"
 
@@ -29,11 +31,17 @@ __device__ __forceinline__ int fx_exp(double v) { return (__double2hiint(v) >> 2
 // above, no denormal results below; everything else goes to the FP64 forms.
 __device__ __forceinline__ bool fx_range(int e) { return e >= 128 && e <= 1900; }
 
-// The leading bit of a number of the block's largest exponent: kFxTop for the
-// equilibrium's monomials (at most 180 of them in one value, counted with
-// their factors) and for the non-equilibrium moments (at most 152), kFxSum for
-// the sums of populations (at most 52, in sum g c), so that all stay below 2^63.
-constexpr int kFxTop = 54, kFxSum = 56;
+// The leading bit of a number of the block's largest exponent.  kFxTop: the
+// non-equilibrium moments (at most 152 in one value, counted with their
+// factors, which stays below 2^63) and the base of the equilibrium's unit.
+// fx_top: the sums of populations.  With 56 of them the operands' rounding was
+// of the size of the stored populations' own (D2Q37: velocities of a decaying
+// pulse 20 % further off than with FP64 sums).  D2Q9 and D2Q17 have room for 57
+// in 64 bits (at most 20 populations in one sum, counted with c); D2Q37 (52)
+// takes 58 and adds its per-speed sums (at most 14 each) in 128 bits.
+constexpr int kFxTop = 54;
+template <int LAT>
+constexpr int fx_top() { return Lat<LAT>::Q > 17 ? 58 : 57; }
 
 // v in units of 2^(emax - 1023 - T), rounded to nearest (truncation is a
 // drift that adds up over the steps); |v| < 2^(emax - 1022), emax >= 128.
@@ -48,15 +56,16 @@ __device__ __forceinline__ long long fx_of(double v, int emax)
     return (a ^ s) - s;
 }
 
-// The same for T = kFxTop with 32 more bits below, truncated.
+// The same for T = kFxTop with 32 more bits below, truncated; |v| < 2^(emax - 1014).
 __device__ __forceinline__ __int128 fx_wide_of(double v, int emax)
 {
     const int hi = __double2hiint(v);
     const unsigned long long m =
         (unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v);
-    // m << (32 + kFxTop - 52 - d) as high and low words
-    const int d = emax - ((hi >> 20) & 0x7ff), n = d < 95 ? d : 95;
-    unsigned long long h = m >> (64 - 32 - (kFxTop - 52)), l = m << (32 + kFxTop - 52);
+    // m << (32 + kFxTop - 52 - d) as high and low words, eight places higher first
+    constexpr int UP = 32 + kFxTop - 52 + 8;
+    const int d = emax - ((hi >> 20) & 0x7ff) + 8, n = d < 95 ? d : 95;
+    unsigned long long h = m >> (64 - UP), l = m << UP;
     if (n >= 64) {
         l = h >> (n - 64);
         h = 0;
@@ -66,6 +75,34 @@ __device__ __forceinline__ __int128 fx_wide_of(double v, int emax)
     }
     const __int128 a = (__int128)((unsigned __int128)h << 64 | l);
     return hi < 0 ? -a : a;
+}
+
+// c_s^2, its square and its inverse in units of 2^-60: of the double that the
+// moments are formed with, on D2Q9 (isothermal: no moment takes it) of 1/3.
+template <int LAT>
+struct FxCs2 {
+    long long c, cc, inv;
+    constexpr FxCs2() : c(0), cc(0), inv(0)
+    {
+        if (!Lat<LAT>::THERMAL) {
+            c = ((1LL << 60) + 1) / 3;
+            inv = 3LL << 60;
+            return;
+        }
+        double v = Lat<LAT>::CS2;
+        int e = 0;
+        for (; v < 4503599627370496.0; ++e) v *= 2.0;      // c_s^2 = m 2^-e, 2^52 <= m < 2^53
+        const __int128 m = (__int128)v;
+        c = (long long)((m << 60) >> e);
+        cc = (long long)((m * m) >> (2 * e - 60));
+        inv = (long long)((((__int128)1 << (60 + e)) + m / 2) / m);
+    }
+};
+
+// x k 2^-60, |x| < 2^95
+__device__ __forceinline__ __int128 fx_mul(__int128 x, long long k)
+{
+    return ((__int128)(long long)(x >> 32) * k >> 28) + ((__int128)(unsigned)x * k >> 60);
 }
 
 // x units of 2^(emax - 1023 - T) as a double, rounded to nearest.
@@ -80,6 +117,14 @@ __device__ __forceinline__ double fx_double(long long x, int emax)
     const unsigned e = (unsigned)(emax + (63 - T) - 1 - n) << 20;
     const unsigned h = (unsigned)(m >> 32) + e + ((unsigned)s & 0x80000000u);
     return a ? __hiloint2double((int)h, (int)(unsigned)m) : 0.0;
+}
+
+// The same for a sum that may be beyond 63 bits, which drops 8 of them then.
+template <int T>
+__device__ __forceinline__ double fx_double(__int128 x, int emax)
+{
+    const bool big = (long long)(x >> 64) != (long long)x >> 63;
+    return fx_double<T>(big ? (long long)((x + 128) >> 8) : (long long)x, big ? emax + 8 : emax);
 }
 
 // A positive double as a 53-bit integer times a power of two, m 2^e, and the
@@ -142,32 +187,33 @@ template <int LAT, typename Get>
 __device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double& sx, double& sy, double& se)
 {
     using L = Lat<LAT>;
+    constexpr int T = fx_top<LAT>();
     long long E[L::NCLS], X[4] = {0, 0, 0, 0}, Y[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int k = 0; k < L::NCLS; ++k) E[k] = 0;
-    E[0] = fx_of<kFxSum>(get(0), emax);
+    E[0] = fx_of<T>(get(0), emax);
 #pragma unroll
     for (int i = 1; i < L::Q; i += 2) {
         const int cx = L::cx(i), cy = L::cy(i);
-        const long long p = fx_of<kFxSum>(get(i), emax), m = fx_of<kFxSum>(get(i + 1), emax), o = p - m;
+        const long long p = fx_of<T>(get(i), emax), m = fx_of<T>(get(i + 1), emax), o = p - m;
         E[L::cls(i)] += p + m;
         if (cx > 0) X[cx] += o;
         if (cx < 0) X[-cx] -= o;
         if (cy > 0) Y[cy] += o;
         if (cy < 0) Y[-cy] -= o;
     }
-    // the energy's factors (216 in all) beyond 64 bits, rounded to units of 4
-    long long a0 = 0;
-    __int128 ae = 2;
+    using A = std::conditional_t<(T > 57), __int128, long long>;
+    A a0 = 0;
+    __int128 ae = 0;
 #pragma unroll
     for (int k = 0; k < L::NCLS; ++k) {
         a0 += E[k];
         if (L::THERMAL) ae += (__int128)L::c2cls(k) * E[k];
     }
-    s0 = fx_double<kFxSum>(a0, emax);
-    sx = fx_double<kFxSum>(X[1] + 2 * X[2] + 3 * X[3], emax);
-    sy = fx_double<kFxSum>(Y[1] + 2 * Y[2] + 3 * Y[3], emax);
-    se = L::THERMAL ? fx_double<kFxSum - 2>((long long)(ae >> 2), emax) : 0.0;
+    s0 = fx_double<T>(a0, emax);
+    sx = fx_double<T>(X[1] + A(2) * X[2] + A(3) * X[3], emax);
+    sy = fx_double<T>(Y[1] + A(2) * Y[2] + A(3) * Y[3], emax);
+    se = L::THERMAL ? fx_double<T>(ae, emax) : 0.0;
 }
 
 // Moments (Eq. macro) of populations get(i); false if they are out of range.
@@ -186,14 +232,19 @@ __device__ __forceinline__ bool fx_moments(Get&& get, double rho0, int ref, doub
 // The equilibrium (see eq_poly) of moments m held against w rho0, in the
 // monomials of (c_x, c_y):
 //   g^eq_i / w_i = sum over a + b <= ORDER of m_ab c_x^a c_y^b,
-// one value at a time to put(i, w, x, e): g^eq_i = fx_scaled(x, w, e).  False, with nothing put, if
-// the coefficients are out of the fixed-point range.  (jx, jy): the momentum
-// rho u.  All velocities share the coefficients' rounding, which in a uniform
-// stream adds up over the steps, so the linear ones, which carry the
-// momentum, are formed in three parts: the product j / c_s^2, its rounding
-// error, and the small nonlinear rest (drift of u without it: 3e-17 u a step).
+// one value at a time to put(i, w, x, e): g^eq_i = fx_scaled(x, w, e).  False,
+// with nothing put, if the coefficients are out of the fixed-point range.
+// (jx, jy), se: rho u and sum g |c|^2.  All velocities share the coefficients'
+// rounding, which in a uniform stream adds up over the steps; so the ones that
+// carry mass, momentum and energy are not formed in FP64 but closed in the
+// integers, with q = 3 m_40 + 3 m_04 + m_22:
+//   m_20 + m_02 = (se - 2 c_s^2 s) / (2 c_s^4) - 2 c_s^2 q  (thermal lattices),
+//   m_00 = s - c_s^2 (m_20 + m_02) - c_s^4 q,
+//   m_10 = j_x / c_s^2 - c_s^2 (3 m_30 + m_12),  m_01 likewise,
+// which is what the expansion's coefficients are, so that g^eq carries s, j
+// and se whatever the rounding of the others, of 1 / c_s^2, u and theta.
 template <int LAT, typename Put>
-__device__ __forceinline__ bool fx_equilibrium(const Moments<LAT, double>& m, double jx, double jy, Put&& put)
+__device__ __forceinline__ bool fx_equilibrium(const Moments<LAT, double>& m, double jx, double jy, double se, Put&& put)
 {
     using L = Lat<LAT>;
     using W = __int128;
@@ -207,10 +258,9 @@ __device__ __forceinline__ bool fx_equilibrium(const Moments<LAT, double>& m, do
     constexpr int NM = O4 ? 15 : O3 ? 10 : 6;
     double c[NM];
     const double rX = jx * ics2, rY = jy * ics2, XX = X * X, XY = X * Y, YY = Y * Y;
-    const double lX = fma(jx, ics2, -rX), lY = fma(jy, ics2, -rY);
     const double rA2 = m.rho * e.A2, rB0 = m.rho * (e.B0 * ics2);
-    c[0] = m.s0 + m.rho * e.A0;             // 1
-    c[1] = rX;                              // x
+    c[0] = m.s0;                            // 1, without the closing part
+    c[1] = rX;                              // x (its size; the value is closed)
     c[2] = rY;                              // y
     c[3] = rB0 + rA2 * XX;                  // x^2
     c[4] = rB0 + rA2 * YY;                  // y^2
@@ -233,20 +283,40 @@ __device__ __forceinline__ bool fx_equilibrium(const Moments<LAT, double>& m, do
     int ec = 0;
 #pragma unroll
     for (int k = 0; k < NM; ++k) ec = max(ec, fx_exp(c[k]));
+    if (L::THERMAL) ec = max(ec, fx_exp(se));
     if (ec == 0) ec = 1023;                 // all zero
     if (!fx_range(ec)) return false;
+    // the largest value that can arise, in units of 2^(ec - 1022 - 20): the
+    // factors are the monomials' at the outermost velocities, with the closing
+    // parts' shares (c_s^2 < 0.7).  The unit is chosen so that it stays below
+    // 2^63 (seven to minus one bits below that of ec and kFxTop).
+    constexpr int F[15] = {1, 3, 3, 10, 10, 4, 34, 34, 12, 12, 83, 83, 17, 27, 27};
+    int bound = 16;
+#pragma unroll
+    for (int k = 0; k < NM; ++k) bound += (F[k] << 20) >> min(ec - fx_exp(c[k]), 31);
+    if (L::THERMAL) bound += (1 << 20) >> min(ec - fx_exp(se), 31);
+    ec -= __clz(bound) - 4;
+    constexpr FxCs2<LAT> K{};
     W v[NM];
 #pragma unroll
-    for (int k = 0; k < NM; ++k) v[k] = fx_wide_of(c[k], ec);
-    v[1] += fx_wide_of(lX, ec);
-    v[2] += fx_wide_of(lY, ec);
-    if constexpr (O3) {                 // (A1 - 1) of eq_poly
-        const double a1 = fma(-0.5, m.ux * X + m.uy * Y, -2.0 * m.dT);
-        const double nx = rX * a1, ny = rY * a1;
-        if (fx_exp(nx) > ec || fx_exp(ny) > ec) return false;
-        v[1] += fx_wide_of(nx, ec);
-        v[2] += fx_wide_of(ny, ec);
+    for (int k = 3; k < NM; ++k) v[k] = fx_wide_of(c[k], ec);
+    const W s = fx_wide_of(c[0], ec);
+    W q = 0, tr = v[3] + v[4];
+    if constexpr (O4) q = 3 * (v[10] + v[11]) + v[12];
+    if constexpr (L::THERMAL) {
+        const W d = v[3] - v[4];
+        tr = (fx_mul(fx_mul(fx_wide_of(se, ec) - 2 * fx_mul(s, K.c), K.inv), K.inv) >> 1) - 2 * fx_mul(q, K.c);
+        v[3] = (tr + d) >> 1;
+        v[4] = (tr - d) >> 1;
     }
+    v[0] = s - fx_mul(tr, K.c);
+    v[1] = fx_mul(fx_wide_of(jx, ec), K.inv);
+    v[2] = fx_mul(fx_wide_of(jy, ec), K.inv);
+    if constexpr (O3) {
+        v[1] -= fx_mul(3 * v[6] + v[9], K.c);
+        v[2] -= fx_mul(3 * v[7] + v[8], K.c);
+    }
+    if constexpr (O4) v[0] -= fx_mul(q, K.cc);
     // the parts below are rounded to 64 bits by adding this and dropping 32
     const W half = W(1) << 31;
     v[0] += half;
@@ -301,7 +371,7 @@ __device__ __forceinline__ bool fx_equilibrium(const Moments<LAT, double>& m, do
 template <int LAT, typename Get, typename Put>
 __device__ __forceinline__ bool fx_relax(const Moments<LAT, double>& m, double om, Get&& get, Put&& put)
 {
-    return fx_equilibrium<LAT>(m, m.sx, m.sy, [&](int i, FxConst w, long long x, int e) {
+    return fx_equilibrium<LAT>(m, m.sx, m.sy, m.se, [&](int i, FxConst w, long long x, int e) {
         const double g = get(i);
         put(i, fma(om, fx_scaled(x, w, e) - g, g));
     });
