@@ -17,7 +17,6 @@
 // kernel parameter bank).  The FP32/FP16 paths do all of their arithmetic in
 // FP32; the FP64 path in FP64.
 #include "collide.cuh"
-#include "ff.cuh"
 #include "fix64.cuh"
 
 #include <utility>
@@ -595,10 +594,11 @@ __device__ __noinline__ void macros_wide(const Geom& G, const S* in, double* U)
     U[3] = m.dT;
 }
 
-// Macroscopic fields of the stored populations.  With FP32 / FP16 storage the
-// sums are float-float (macros_ff).  As FP64 sums (about 200 FP64
+// Macroscopic fields of the stored populations, their sums in block fixed
+// point (fix64.cuh): exact for FP32 and FP16 populations within 2^33 of the
+// node's largest, with one rounding to FP64 each.  As FP64 sums (about 200 FP64
 // instructions a node, 64 cycles a warp instruction) the kernel was bound by
-// the FP64 pipe: D2Q37 4096^2 with FP32 storage 6.19 ms, now 0.82 ms; the
+// the FP64 pipe: D2Q37 4096^2 with FP32 storage 6.19 ms, now 0.72 ms (FP16 0.83); the
 // 3.0 GB it moves take 0.44 ms at the measured copy bandwidth.
 template <int LAT, typename S>
 __global__ void __launch_bounds__(kBulkThreads) k_macros(Geom G, const S* __restrict__ f, double* __restrict__ rho,
@@ -622,8 +622,25 @@ __global__ void __launch_bounds__(kBulkThreads) k_macros(Geom G, const S* __rest
         float h[L::Q];
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) h[i] = Store<S>::load(in + (long long)L::plane_of(i) * G.plane);
-        macros_ff<LAT, S>(G, h, U);
-        if (!finite()) macros_wide<LAT, S>(G, in, U);   // beyond the float range
+        double s0, sx, sy, se;
+        bool ok;
+        if constexpr (Store<S>::SCALED) {
+            ok = fx_sums_scaled<LAT>(h, s0, sx, sy, se);
+        } else {
+            const int emax = fx_block_float<LAT>(h);
+            ok = emax != 0;
+            if (ok) fx_sums<LAT, kFxFloat>([&](int i) { return h[i]; }, emax, s0, sx, sy, se);
+        }
+        if (ok) {
+            const Moments<LAT, double> m =
+                moments_of_sums<LAT, double>(s0, sx, sy, se, G.rho0, G.ref, stored_ref<S>(G, 0), stored_ref<S>(G, 1));
+            U[0] = m.s0;
+            U[1] = m.ux;
+            U[2] = m.uy;
+            U[3] = m.dT;
+        } else {
+            macros_wide<LAT, S>(G, in, U);
+        }
     } else {
         double g[L::Q];
 #pragma unroll

@@ -39,7 +39,8 @@ __device__ __forceinline__ bool fx_range(int e) { return e >= 128 && e <= 1900; 
 // pulse 20 % further off than with FP64 sums).  D2Q9 and D2Q17 have room for 57
 // in 64 bits (at most 20 populations in one sum, counted with c); D2Q37 (52)
 // takes 58 and adds its per-speed sums (at most 14 each) in 128 bits.
-constexpr int kFxTop = 54;
+// kFxFloat: the sums of FP32 populations (52 of them in 64 bits).
+constexpr int kFxTop = 54, kFxFloat = 56;
 template <int LAT>
 constexpr int fx_top() { return Lat<LAT>::Q > 17 ? 58 : 57; }
 
@@ -54,6 +55,18 @@ __device__ __forceinline__ long long fx_of(double v, int emax)
     const int d = emax - ((hi >> 20) & 0x7ff);
     const long long a = (long long)(((m >> (d < 63 ? d : 63)) + 1) >> 1), s = hi >> 31;
     return (a ^ s) - s;
+}
+
+// A float in the same units, rounded down (the sums of a read-out feed nothing
+// back): exact if its last bit is above the unit.  Denormals count as zero;
+// a block of them (fx_block_float) goes to the FP64 form.
+template <int T>
+__device__ __forceinline__ long long fx_of(float v, int emax)
+{
+    const int b = __float_as_int(v), s = b >> 31, e = (b >> 23) & 0xff;
+    const int m = e ? (((b & 0x7fffff) | 0x800000) ^ s) - s : 0;
+    const int d = emax - (1023 - 127) + (62 - T) - e;
+    return (long long)((unsigned long long)(unsigned)m << 39) >> (d < 63 ? d : 63);
 }
 
 // The same for T = kFxTop with 32 more bits below, truncated; |v| < 2^(emax - 1014).
@@ -182,12 +195,23 @@ __device__ __forceinline__ int fx_block(Get&& get)
     return any == 0 ? 1023 : fx_range(emax) ? emax : 0;
 }
 
+// The same of FP32 populations: zeros and values of 2^-67 to the
+// largest, so that a denormal is below the unit.
+template <int LAT>
+__device__ __forceinline__ int fx_block_float(const float* g)
+{
+    int emax = 0;
+#pragma unroll
+    for (int i = 0; i < Lat<LAT>::Q; ++i) emax = max(emax, __float_as_int(g[i]) & 0x7fffffff);
+    const int e = emax >> 23;
+    return emax == 0 ? 1023 : e >= 60 && e < 255 ? e + (1023 - 127) : 0;
+}
+
 // The sums of Eq. macro: s0 = sum g, (sx, sy) = sum g c, se = sum g |c|^2.
-template <int LAT, typename Get>
+template <int LAT, int T = fx_top<LAT>(), typename Get>
 __device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double& sx, double& sy, double& se)
 {
     using L = Lat<LAT>;
-    constexpr int T = fx_top<LAT>();
     long long E[L::NCLS], X[4] = {0, 0, 0, 0}, Y[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int k = 0; k < L::NCLS; ++k) E[k] = 0;
@@ -214,6 +238,82 @@ __device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double&
     sx = fx_double<T>(X[1] + A(2) * X[2] + A(3) * X[3], emax);
     sy = fx_double<T>(Y[1] + A(2) * Y[2] + A(3) * Y[3], emax);
     se = L::THERMAL ? fx_double<T>(ae, emax) : 0.0;
+}
+
+// x 2^-88 as a double.
+__device__ __forceinline__ double fx_double_scaled(__int128 x)
+{
+    const long long h = (long long)(x >> 64);
+    const int n = 65 - __clzll(h ^ (h >> 63));      // one place more than the high word's bits, and
+    const bool wide = h != (long long)x >> 63;      // none if the low word holds the number
+    return fx_double<88>(wide ? (long long)(x >> n) : (long long)x, wide ? 1023 + n : 1023);
+}
+
+// The same sums of FP16 storage, h = g / w (FP16 values in float); false if
+// one is not finite.  An FP16 value is an integer of 41 bits times 2^-24: two
+// floats, hi 2^-4 + lo 2^-24, whose sums over a class (16 counted with c) are
+// exact in FP32; then the classes' weights in units of 2^-64 (a double's last
+// bit or 2^-65) on 32-bit parts, and one rounding each.
+template <int LAT>
+__device__ __forceinline__ bool fx_sums_scaled(const float* h, double& s0, double& sx, double& sy, double& se)
+{
+    using L = Lat<LAT>;
+    constexpr int N = L::NCLS;
+    float E[N][2], X[N][2], Y[N][2];
+#pragma unroll
+    for (int k = 0; k < N; ++k) E[k][0] = E[k][1] = X[k][0] = X[k][1] = Y[k][0] = Y[k][1] = 0.0f;
+    auto split = [](float v, float* p) {
+        p[0] = fmaf(v, 16.0f, 12582912.0f) - 12582912.0f;       // to an integer (1.5 2^23)
+        p[1] = fmaf(p[0], -1048576.0f, v * 16777216.0f);
+    };
+    split(h[0], E[0]);
+#pragma unroll
+    for (int i = 1; i < L::Q; i += 2) {
+        const int k = L::cls(i);
+        const float cx = float(L::cx(i)), cy = float(L::cy(i));
+        float p[2], m[2];
+        split(h[i], p);
+        split(h[i + 1], m);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            E[k][q] += p[q] + m[q];
+            if (L::cx(i)) X[k][q] = fmaf(cx, p[q] - m[q], X[k][q]);
+            if (L::cy(i)) Y[k][q] = fmaf(cy, p[q] - m[q], Y[k][q]);
+        }
+    }
+    // (hi 2^20 + lo) (wh 2^32 + wl): four sums of 32-bit products each
+    struct Sum {
+        long long a = 0, b = 0, c = 0, d = 0;
+        __device__ void add(int hi, int lo, long long w)
+        {
+            const int wl = int(unsigned(w)), wh = int((w - wl) >> 32);
+            a += (long long)hi * wh;
+            b += (long long)hi * wl;
+            c += (long long)lo * wh;
+            d += (long long)lo * wl;
+        }
+        __device__ double get() const
+        {
+            return fx_double_scaled((((__int128)a << 20) + c << 32) + ((__int128)b << 20) + d);
+        }
+    } S, SX, SY, SE;
+    float all = 0.0f;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const long long w = (long long)(L::wcls(k) * 18446744073709551616.0);     // below 1/2
+        all += E[k][1];
+        const int hi = __float2int_rn(E[k][0]), lo = __float2int_rn(E[k][1]);
+        S.add(hi, lo, w);
+        if (k == 0) continue;
+        if (L::THERMAL) SE.add(hi, lo, L::c2cls(k) * w);
+        SX.add(__float2int_rn(X[k][0]), __float2int_rn(X[k][1]), w);
+        SY.add(__float2int_rn(Y[k][0]), __float2int_rn(Y[k][1]), w);
+    }
+    s0 = S.get();
+    sx = SX.get();
+    sy = SY.get();
+    se = L::THERMAL ? SE.get() : 0.0;
+    return isfinite(all);               // an infinity leaves NaN in lo
 }
 
 // Moments (Eq. macro) of populations get(i); false if they are out of range.
