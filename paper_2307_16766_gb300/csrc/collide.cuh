@@ -68,7 +68,9 @@ __device__ __forceinline__ Moments<LAT, C> moments_G(const Geom& G, const C* g)
 // runs: 30.5, 29.8), and the gradients of short runs feel its different
 // rounding.  FP16 storage and populations relative to a reference, where
 // there are no gradients, take the closed form: 1024x512 with a reference 3.87 ms
-// a pass (4.00 with the sums), 4096^2 FP16 11.59 (11.65).
+// a pass (4.00 with the sums); FP16, 60 steps: 512x512 with an outlet 1.43 ms
+// (1.53), 1024x512 with four sides 1.92 (2.03), 1600x1200 4.84 (4.91), 2048^2
+// 9.06 (9.08).
 template <int LAT, typename C, typename T>
 __device__ __forceinline__ void neq_evaluated(const C* g, const Moments<LAT, C>& m, T fac, T* N)
 {
@@ -191,6 +193,34 @@ __device__ __forceinline__ void neq_close(const Moments<LAT, C>& m, T fac, T* N,
     }
 }
 
+// The elements at(0..Q-1) points to, as values.  FP16: the raw words of all of
+// them first (the empty asm statements hold them), then the conversions; as
+// one loop each load was waited for before the next (k_band with FP16 storage,
+// D2Q37 512x512: 40 us a step, 23 us with the loads in flight together, FP32 21).
+template <int LAT, typename S, typename C, bool LIVE, typename At>
+__device__ __forceinline__ void load_all(At&& at, C* g)
+{
+    constexpr int Q = Lat<LAT>::Q;
+    if constexpr (sizeof(S) == 2) {
+        unsigned r[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const unsigned short* p = reinterpret_cast<const unsigned short*>(at(i));
+            r[i] = LIVE ? *p : __ldg(p);
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) asm volatile("" : "+r"(r[i]));
+#pragma unroll
+        for (int i = 0; i < Q; ++i) g[i] = C(Store<S>::value(__ushort_as_half((unsigned short)r[i])));
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            if constexpr (LIVE) g[i] = C(Store<S>::value(*at(i)));
+            else g[i] = C(Store<S>::load(at(i)));
+        }
+    }
+}
+
 // Plain pull of node (x, y) with periodic wrap-around of the sources.  LIVE:
 // the previous step may still have been writing fin when this kernel started
 // (early start), so the loads are ordinary ones, which the wait for that step
@@ -200,15 +230,14 @@ template <int LAT, typename S, typename C, bool LIVE = false>
 __device__ __forceinline__ void pull_plain(const Geom& G, const Offsets& O, const S* fin, int x, int y, C* g)
 {
     using L = Lat<LAT>;
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        int xs = x - L::cx(i), ys = y - L::cy(i);
-        if (L::cx(i) && G.perx) xs = xs < 0 ? xs + G.nx : (xs >= G.nx ? xs - G.nx : xs);
-        if (L::cy(i) && G.pery) ys = ys < 0 ? ys + G.ny : (ys >= G.ny ? ys - G.ny : ys);
-        const S* p = fin + (O.st[i] + ys * G.nxp + xs);
-        if constexpr (LIVE) g[i] = C(Store<S>::value(*p));
-        else g[i] = C(Store<S>::load(p));
-    }
+    load_all<LAT, S, C, LIVE>(
+        [&](int i) {
+            int xs = x - L::cx(i), ys = y - L::cy(i);
+            if (L::cx(i) && G.perx) xs = xs < 0 ? xs + G.nx : (xs >= G.nx ? xs - G.nx : xs);
+            if (L::cy(i) && G.pery) ys = ys < 0 ? ys + G.ny : (ys >= G.ny ? ys - G.ny : ys);
+            return fin + (O.st[i] + ys * G.nxp + xs);
+        },
+        g);
 }
 
 // The same with the plane offsets computed from the plane size (for kernels
@@ -219,13 +248,14 @@ __device__ __forceinline__ void pull_plain_planes(const Geom& G, const S* __rest
 {
     using L = Lat<LAT>;
     const int plane = int(G.plane);
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-        int xs = x - L::cx(i), ys = y - L::cy(i);
-        if (L::cx(i) && G.perx) xs = xs < 0 ? xs + G.nx : (xs >= G.nx ? xs - G.nx : xs);
-        if (L::cy(i) && G.pery) ys = ys < 0 ? ys + G.ny : (ys >= G.ny ? ys - G.ny : ys);
-        g[i] = C(Store<S>::load(fin + (L::plane_of(i) * plane + ys * G.nxp + xs)));
-    }
+    load_all<LAT, S, C, false>(
+        [&](int i) {
+            int xs = x - L::cx(i), ys = y - L::cy(i);
+            if (L::cx(i) && G.perx) xs = xs < 0 ? xs + G.nx : (xs >= G.nx ? xs - G.nx : xs);
+            if (L::cy(i) && G.pery) ys = ys < 0 ? ys + G.ny : (ys >= G.ny ? ys - G.ny : ys);
+            return fin + (L::plane_of(i) * plane + ys * G.nxp + xs);
+        },
+        g);
 }
 
 // Moments (Eq. macro) and BGK collision (Eq. bgk) of one node whose pulled
