@@ -627,9 +627,10 @@ __global__ void __launch_bounds__(kBulkThreads) k_macros(Geom G, const S* __rest
         if constexpr (Store<S>::SCALED) {
             ok = fx_sums_scaled<LAT>(h, s0, sx, sy, se);
         } else {
-            const int emax = fx_block_float<LAT>(h);
+            int lift;
+            const int emax = fx_block_float<LAT>(h, lift);
             ok = emax != 0;
-            if (ok) fx_sums<LAT, kFxFloat>([&](int i) { return h[i]; }, emax, s0, sx, sy, se);
+            if (ok) fx_sums<LAT, kFxFloat>([&](int i) { return h[i]; }, emax, s0, sx, sy, se, lift);
         }
         if (ok) {
             const Moments<LAT, double> m =

@@ -58,8 +58,8 @@ __device__ __forceinline__ long long fx_of(double v, int emax)
 }
 
 // A float in the same units, rounded down (the sums of a read-out feed nothing
-// back): exact if its last bit is above the unit.  Denormals count as zero;
-// a block of them (fx_block_float) goes to the FP64 form.
+// back): exact if its last bit is above the unit.  Denormals count as zero
+// (fx_block_float).
 template <int T>
 __device__ __forceinline__ long long fx_of(float v, int emax)
 {
@@ -195,21 +195,32 @@ __device__ __forceinline__ int fx_block(Get&& get)
     return any == 0 ? 1023 : fx_range(emax) ? emax : 0;
 }
 
-// The same of FP32 populations: zeros and values of 2^-67 to the
-// largest, so that a denormal is below the unit.
+// The same of FP32 populations: 0 only for infinities and NaN.  A block below
+// 2^-67 (the front of a pulse) is lifted by 2^lift first, so that denormals
+// count in it; in the others they are below the unit.
 template <int LAT>
-__device__ __forceinline__ int fx_block_float(const float* g)
+__device__ __forceinline__ int fx_block_float(float* g, int& lift)
 {
     int emax = 0;
+    lift = 0;
 #pragma unroll
     for (int i = 0; i < Lat<LAT>::Q; ++i) emax = max(emax, __float_as_int(g[i]) & 0x7fffffff);
+    if (emax == 0) return 1023;
+    if (emax < 60 << 23) {
+        lift = 96;
+#pragma unroll
+        for (int i = 0; i < Lat<LAT>::Q; ++i) g[i] *= 7.9228162514264338e28f;
+        emax = __float_as_int(__int_as_float(emax) * 7.9228162514264338e28f);
+    }
     const int e = emax >> 23;
-    return emax == 0 ? 1023 : e >= 60 && e < 255 ? e + (1023 - 127) : 0;
+    return e < 255 ? e + (1023 - 127) : 0;
 }
 
-// The sums of Eq. macro: s0 = sum g, (sx, sy) = sum g c, se = sum g |c|^2.
+// The sums of Eq. macro: s0 = sum g, (sx, sy) = sum g c, se = sum g |c|^2, of
+// populations lifted by 2^lift.
 template <int LAT, int T = fx_top<LAT>(), typename Get>
-__device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double& sx, double& sy, double& se)
+__device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double& sx, double& sy, double& se,
+                                        int lift = 0)
 {
     using L = Lat<LAT>;
     long long E[L::NCLS], X[4] = {0, 0, 0, 0}, Y[4] = {0, 0, 0, 0};
@@ -234,6 +245,7 @@ __device__ __forceinline__ void fx_sums(Get&& get, int emax, double& s0, double&
         a0 += E[k];
         if (L::THERMAL) ae += (__int128)L::c2cls(k) * E[k];
     }
+    emax -= lift;
     s0 = fx_double<T>(a0, emax);
     sx = fx_double<T>(X[1] + A(2) * X[2] + A(3) * X[3], emax);
     sy = fx_double<T>(Y[1] + A(2) * Y[2] + A(3) * Y[3], emax);
