@@ -330,9 +330,10 @@ typedef struct lbm_batch lbm_batch;
  * all its runs and one persistent bulk launch whose CTAs loop over the row
  * segments of all its runs; after the first two steps each parity's step
  * is captured once as a CUDA graph and replayed.  The persistent kernel's
- * CTAs per SM are autotuned on the first step (fastest of 1..5) and cached
- * per device, lattice, storage and size bucket in the text file named by
- * the environment variable LBM_AUTOTUNE_CACHE (default
+ * CTAs per SM are autotuned on the first step (fastest of 1..5 over whole
+ * steps) and cached per device and make-up of the batch (of each lattice and
+ * storage the sizes of the bulk work and of the band, as powers of two) in
+ * the text file named by the environment variable LBM_AUTOTUNE_CACHE (default
  * ~/.cache/lbm_cbc_autotune.txt; an empty value turns the cache off).  At
  * most 256 runs per lattice and storage.  Allocates with cudaMalloc. */
 int lbm_batch_create(int n, const int* lattice, const int* nx, const int* ny, const double* tau,

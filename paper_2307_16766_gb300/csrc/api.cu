@@ -1744,8 +1744,12 @@ int batch_fail(lbm_batch* b, cudaError_t e, const char* what)
 
 // Autotuned CTAs per SM of the persistent bulk kernel, cached in a text file
 // (LBM_AUTOTUNE_CACHE, default ~/.cache/lbm_cbc_autotune.txt; empty = off):
-// one line "device lattice storage bucket ctas_per_sm" per tuned case, the
-// bucket being log2 of the group's work items.
+// one line "step device groups group ctas_per_sm" per tuned group.  What is
+// timed is a whole step, so the key holds all that runs in it: of every group
+// of the batch, in the order they are tuned in, lattice.storage.items.tiles
+// (work items of the bulk kernel and band tiles, as log2 and one more, 0 for
+// none), and the place of the tuned one among them.  ("step": entries of the
+// library that timed the bulk kernel alone begin with the device.)
 std::string autotune_path()
 {
     const char* p = getenv("LBM_AUTOTUNE_CACHE");
@@ -1754,7 +1758,7 @@ std::string autotune_path()
     return home ? std::string(home) + "/.cache/lbm_cbc_autotune.txt" : std::string();
 }
 
-std::string autotune_key(int lattice, int storage, int items)
+std::string autotune_key(const std::vector<lbm_batch::Group>& groups, size_t which)
 {
     int dev = 0;
     cudaDeviceProp prop;
@@ -1763,9 +1767,15 @@ std::string autotune_key(int lattice, int storage, int items)
     std::string name = prop.name;
     for (char& c : name)
         if (c == ' ') c = '_';
-    int bucket = 0;
-    while ((1 << bucket) < items) ++bucket;
-    return fmt("%s %d %d %d", name.c_str(), lattice, storage, bucket);
+    auto bucket = [](int n) {
+        int b = 0;
+        while (n > 0 && (1LL << b) < n) ++b;
+        return n > 0 ? b + 1 : 0;
+    };
+    std::string all;
+    for (const auto& g : groups)
+        all += fmt("%s%d.%d.%d.%d", all.empty() ? "" : "/", g.lattice, g.storage, bucket(g.total_items), bucket(g.n_tiles));
+    return fmt("step %s %s %d", name.c_str(), all.c_str(), int(which));
 }
 
 int autotune_lookup(const std::string& key)
@@ -1856,8 +1866,9 @@ int batch_autotune(lbm_batch* b)
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e != cudaSuccess) return batch_fail(b, e, "autotune events");
     const int par = int(b->steps & 1);
-    for (auto& g : b->groups) {
-        const std::string key = autotune_key(g.lattice, g.storage, g.total_items);
+    for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+        lbm_batch::Group& g = b->groups[gi];
+        const std::string key = autotune_key(b->groups, gi);
         int best = autotune_lookup(key);
         if (!best) {
             float best_ms = 1e30f;
