@@ -185,17 +185,18 @@ def bulk_traffic(storage, launch_nodes):
 def bulk_fp64_flops():
     """FP64 flops per node update of k_bulk<D2Q37, double> (2 per FMA, 1 per
     add or multiply) from the committed ncu counter capture, if it was taken
-    on the current sources of the kernel (bulk.cu and collide.cuh)."""
-    h = hashlib.sha256()
-    for f in ("bulk.cu", "collide.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2307_16766_gb300", "csrc", f), "rb").read())
-    sha = h.hexdigest()[:12]
+    on the current sources of the kernel (src: bulk.cu and collide.cuh) and of
+    its arithmetic (arith: fix64.cuh and lbm_internal.cuh)."""
+    sha, arith = (hashlib.sha256(b"".join(open(os.path.join(ROOT, "paper_2307_16766_gb300", "csrc", f), "rb").read()
+                                          for f in files)).hexdigest()[:12]
+                  for files in (("bulk.cu", "collide.cuh"), ("fix64.cuh", "lbm_internal.cuh")))
     path = os.path.join(ROOT, "profiles", "k_bulk_d2q37_f64_flops.txt")
     if not os.path.exists(path):
         return None
     for line in open(path):
-        m = re.match(r"flops\s+nodes=(\d+)\s+dfma=(\d+)\s+dadd=(\d+)\s+dmul=(\d+)\s+src=(\w+)", line.strip())
-        if m and m.group(5) == sha:
+        m = re.match(r"flops\s+nodes=(\d+)\s+dfma=(\d+)\s+dadd=(\d+)\s+dmul=(\d+)\s+src=(\w+)\s+arith=(\w+)",
+                     line.strip())
+        if m and m.group(5) == sha and m.group(6) == arith:
             n, fma, add, mul = (int(m.group(k)) for k in range(1, 5))
             return {"flops": (2 * fma + add + mul) / n, "instructions": (fma + add + mul) / n}
     return None
