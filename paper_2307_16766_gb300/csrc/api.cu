@@ -1040,7 +1040,8 @@ int lbm_step(lbm_handle* h, int n)
         bool early = i > 0 && !timed && h->B.n_zg == 0;
         if (h->B.n_tiles == 0) {
             // no characteristic side: bulk, inflow and zero gradient in order
-            // (no early start after an inflow kernel)
+            // (no early start while an inflow kernel is still to come; right
+            // after one the wait is for that kernel, which is stream-ordered)
             if (h->n_inflow > 0 && !(h->inflow_done[0] && h->inflow_done[1])) early = false;
             rc = bulk(h, par, h->stream, early && !h->G.ref ? CHAIN_BULK : CHAIN_NONE);
             if (rc == LBM_OK) rc = band(h, par, h->stream);

@@ -8,9 +8,9 @@
 //            populations (equilibrium or Eq. NEEP) post-collision.
 //  k_zg      zero-gradient copies (Eq. zg-bc), after the bulk update.
 //
-// The characteristic decomposition and the RK4 update are FP64; with FP32
-// or FP16 storage the fused kernel forms their inputs (stencils,
-// transversal and viscous terms, strip macros) in FP32.  Every neighbour a
+// The characteristic decomposition and the RK4 update are FP64 with FP64
+// storage and float-float with FP32 or FP16 storage, where their inputs
+// (stencils, transversal and viscous terms, strip macros) are FP32.  Every neighbour a
 // right-hand side needs is resolved on the host into a UDesc: another
 // unknown (stage value) or a strip node holding a bulk node's macros at t
 // and t + 1 (interpolated linearly at the stage time, Sec. 3.3).
@@ -227,11 +227,6 @@ __device__ __forceinline__ bool wait_exchange(unsigned long long* bar, unsigned 
         }
     }
 }
-
-__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
-__device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
 
 // S row products, RK4 sums and frames in float-float, for the one-CTA tile.
 __device__ __forceinline__ FF ff_addf(FF x, float b)
@@ -587,13 +582,11 @@ __device__ __forceinline__ void band_tile_mono(const Geom& G, const Offsets& O, 
 //    unknowns by level: level 0 are owned, level l computes the first 4 - l
 //    stages, level 4 only supplies U(t).  Per stage, the inputs of the
 //    characteristic system (1/rho, sqrt(theta), 1/sqrt(theta), P - P_inf
-//    and the transversal terms; in type R), then wave r, then lab component
-//    r of the right-hand side and of the stage value (float-float with
-//    FP32 / FP16 storage, FP64 with FP64 storage; stage values are shared in
-//    type R).  Stage 0 freezes the viscous vector and the incoming-wave
+//    and the transversal terms), then wave r, then lab component r of the
+//    right-hand side and of the stage value.  Stage 0 freezes the viscous vector and the incoming-wave
 //    mask of time t.
 // 3. The owners write U(t + 1) and the mesoscopic Dirichlet populations
-//    (equilibrium or Eq. NEEP), shared out over the four groups.
+//    (equilibrium or Eq. NEEP), shared out over the four CTAs.
 template <int LAT, typename S, bool REF, bool BATCH>
 __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const Band& B,
                                           const Export& E, const S* fin,
@@ -838,9 +831,9 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
                 switch (i) {
                 case 0: return R(1) / (rho0r + Ul[0]);
                 case 1: return corner ? R(0) : R(-0.5) * ((rho0r + Up[0]) * Up[2] - (rho0r + Um[0]) * Um[2]);
-                case 2: return TH ? sqrt_r(R(1) + Ul[3]) : R(0);
+                case 2: return TH ? sqrt(R(1) + Ul[3]) : R(0);
                 case 3: return corner ? R(0) : -Ul[2] * (R(0.5) * (Up[1] - Um[1]));
-                case 4: return TH ? rsqrt_r(R(1) + Ul[3]) : R(0);
+                case 4: return TH ? rsqrt(R(1) + Ul[3]) : R(0);
                 case 5: {
                     const R dP = TH ? cs2r * (Ul[0] + rho0r * Ul[3] + Ul[0] * Ul[3]) : cs2r * Ul[0];
                     return corner ? R(0) : dP - bconst<R>(B.pdev[kind], B.pdev_f[kind]);

@@ -14,8 +14,9 @@
 // segments per CTA with FP32 / FP16 storage (one with the reference
 // equilibrium and with FP64 storage); stores
 // go straight to global memory at fixed plane offsets (Offsets, in the
-// kernel parameter bank).  The FP32/FP16 paths do all of their arithmetic in
-// FP32; the FP64 path in FP64.
+// kernel parameter bank).  The FP32/FP16 updates do all of their arithmetic in
+// FP32; the FP64 update its sums and the equilibrium's monomials in block fixed
+// point (fix64.cuh), the rest in FP64.
 #include "collide.cuh"
 #include "fix64.cuh"
 
@@ -709,11 +710,12 @@ int bulk_t(const Geom& G, const Offsets& O, const Region& R, const CUtensorMap* 
     constexpr size_t smem = ROWS * Stage<LAT, S>::TOTAL;
     static_assert(smem <= 48 * 1024, "bulk staging above the default dynamic shared memory");
     const dim3 grd(t1 - t0, (h + ROWS - 1) / ROWS);
-    if (sizeof(S) == 8 || follow)
-        return launch_ex(k_bulk_chain<LAT, S>, grd, blk, smem, st, chain != CHAIN_NONE, tm, G, O, R,
-                         static_cast<const S*>(fin), static_cast<S*>(fout), status, chain, par);
-    return launch_ex(k_bulk<LAT, S>, grd, blk, smem, st, chain == CHAIN_BAND, tm, G, O, R,
-                     static_cast<const S*>(fin), static_cast<S*>(fout), status);
+    if constexpr (sizeof(S) != 8)
+        if (!follow)
+            return launch_ex(k_bulk<LAT, S>, grd, blk, smem, st, chain == CHAIN_BAND, tm, G, O, R,
+                             static_cast<const S*>(fin), static_cast<S*>(fout), status);
+    return launch_ex(k_bulk_chain<LAT, S>, grd, blk, smem, st, chain != CHAIN_NONE, tm, G, O, R,
+                     static_cast<const S*>(fin), static_cast<S*>(fout), status, chain, par);
 }
 
 template <int LAT, typename S>

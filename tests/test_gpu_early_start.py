@@ -35,3 +35,31 @@ def test_many_steps_in_one_call_equal_one_step_a_call(lattice, nx, ny, storage, 
     a.macros()                              # no kernel gave a wait up
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("storage,sides", [("f64", CBC), ("f64", ("periodic",) * 4), ("f32", ("periodic",) * 4)])
+def test_captured_steps_equal_eager_ones(storage, sides):
+    """Four steps captured in a graph (all but the first with early start) and
+    replayed."""
+    import numpy as np
+    import torch
+    import paper_2307_16766_gb300 as lbm
+    cfg = W.run("D2Q37", 260, 120, 0.8, storage=storage, sides=sides, schemes=("cbc_relax",) * 4, alpha_T=0.4)
+    f = W.smooth_random(260, 120, seed=9, amp=1e-3, u0=(0.03, 0.01))
+    a = lbm.Simulation(cfg).init_fields(*f).step(4 * 25)
+    want = a.macros()
+    a.close()
+    b = lbm.Simulation(cfg).init_fields(*f)
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        lbm.lbm_set_stream(b.handle, s.cuda_stream)
+        lbm.lbm_step(b.handle, 4)
+    for _ in range(25):
+        g.replay()
+    torch.cuda.synchronize()
+    lbm.lbm_set_stream(b.handle, torch.cuda.current_stream().cuda_stream)
+    got = b.macros()
+    b.close()
+    for x, y in zip(want, got):
+        assert np.array_equal(x, y)
