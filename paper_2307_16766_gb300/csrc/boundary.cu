@@ -696,7 +696,8 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
         // are in its range
         Moments<LAT, C> m;
         auto get = [&](int i) { return g[i]; };
-        const int emax = fx_block<LAT>(get);
+        int up;
+        const int emax = fx_block<LAT>(get, up);
         if (!emax || !fx_moments<LAT>(get, G.rho0, REF ? G.ref : 0, G.uref[0], G.uref[1], m))
             m = moments_G<LAT, C, REF>(G, g);
         if (N.fx >= 0) {
@@ -720,7 +721,7 @@ __device__ __forceinline__ void band_tile(const Geom& G, const Offsets& O, const
                 const R fac = R(1) - R(0.5) * omega_of<R>(G);
                 if (emax) {
                     R pxy, dxy, pxx, pyy, rx, ry;
-                    fx_neq_sums<LAT>(get, emax, pxy, dxy, pxx, pyy, rx, ry);
+                    fx_neq_sums<LAT>(get, emax, up, pxy, dxy, pxx, pyy, rx, ry);
                     neq_close<LAT, C, R>(m, fac, N1, pxy, dxy, pxx, pyy, rx, ry);
                 } else {
                     neq_moments<LAT, C, R>(g, m, fac, N1);

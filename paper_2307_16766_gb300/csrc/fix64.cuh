@@ -32,8 +32,9 @@ __device__ __forceinline__ int fx_exp(double v) { return (__double2hiint(v) >> 2
 __device__ __forceinline__ bool fx_range(int e) { return e >= 128 && e <= 1900; }
 
 // The leading bit of a number of the block's largest exponent.  kFxTop: the
-// non-equilibrium moments (at most 152 in one value, counted with their
-// factors, which stays below 2^63) and the base of the equilibrium's unit.
+// base of the units of the non-equilibrium moments (up to 259 populations in
+// one value, counted with their factors) and of the equilibrium, which follow
+// the size of the values (fx_block, fx_equilibrium).
 // fx_top: the sums of populations.  With 56 of them the operands' rounding was
 // of the size of the stored populations' own (D2Q37: velocities of a decaying
 // pulse 20 % further off than with FP64 sums).  D2Q9 and D2Q17 have room for 57
@@ -192,6 +193,41 @@ __device__ __forceinline__ int fx_block(Get&& get)
         any |= unsigned(hi) | unsigned(__double2loint(v));
     }
     emax >>= 20;
+    return any == 0 ? 1023 : fx_range(emax) ? emax : 0;
+}
+
+// The same, and in `up` how many bits further down than kFxTop the sums of
+// fx_neq_sums may go: per class the largest weight a moment's sum gives it in
+// all, with the class's own exponent, stays below 2^63 then (2^-20 of the
+// block's binade a unit of the bound; 54 + up between 53 and 61).
+template <int LAT, typename Get>
+__device__ __forceinline__ int fx_block(Get&& get, int& up)
+{
+    using L = Lat<LAT>;
+    int top[L::NCLS];
+    unsigned any = 0;
+#pragma unroll
+    for (int k = 0; k < L::NCLS; ++k) top[k] = 0;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const double v = get(i);
+        const int hi = __double2hiint(v) & 0x7fffffff;
+        top[L::cls(i)] = max(top[L::cls(i)], hi);
+        any |= unsigned(hi) | unsigned(__double2loint(v));
+    }
+    int emax = 0;
+#pragma unroll
+    for (int k = 0; k < L::NCLS; ++k) {
+        top[k] >>= 20;
+        emax = max(emax, top[k]);
+    }
+    // sum over a class of |c_x c_y|, |c_x^2 - c_y^2|, |c_x^2|, |(|c|^2 - 5) c_x|, |(|c|^2 - 4 c_s^2) c_x|
+    constexpr int W37[8] = {0, 8, 12, 16, 27, 42, 38, 116}, W17[5] = {0, 8, 12, 52, 45}, W9[3] = {0, 2, 4};
+    int bound = 16;
+#pragma unroll
+    for (int k = 1; k < L::NCLS; ++k)
+        bound += ((L::Q == 37 ? W37[k % 8] : L::Q == 17 ? W17[k % 5] : W9[k % 3]) << 20) >> min(emax - top[k], 31);
+    up = min(__clz(bound) - 4, 7);
     return any == 0 ? 1023 : fx_range(emax) ? emax : 0;
 }
 
@@ -491,17 +527,23 @@ __device__ __forceinline__ bool fx_relax(const Moments<LAT, double>& m, double o
 
 // neq_moments (collide.cuh) with its sums in fixed point; get(i) in range.
 // The third moments are sum g (|c|^2 - 5) c + (5 - 4 c_s^2) sum g c, the product
-// with the constant in 128 bits: the two parts all but cancel.
+// with the constant in 128 bits: the two parts all but cancel.  The operands go
+// `up` bits below kFxTop (fx_block; usually three to five).  Without them p_xy
+// was up to 3.5 times, q up to 3.5 times on D2Q17, as far off as the sums over
+// g - g^eq in FP64.
 template <int LAT, typename Get>
-__device__ __forceinline__ void fx_neq_sums(Get&& get, int emax, double& pxy, double& dxy, double& pxx, double& pyy,
-                                            double& rx, double& ry)
+__device__ __forceinline__ void fx_neq_sums(Get&& get, int emax, int up, double& pxy, double& dxy, double& pxx,
+                                            double& pyy, double& rx, double& ry)
 {
     using L = Lat<LAT>;
+    constexpr int T = 61;                       // the finest unit
+    emax -= up;
+    auto of = [&](double v) { return fx_of<T>(v, emax + (T - kFxTop)); };
     long long axy = 0, ad = 0, axx = 0, ayy = 0, ax = 0, ay = 0, jx = 0, jy = 0;
 #pragma unroll
     for (int i = 1; i < L::Q; i += 2) {
         const int cx = L::cx(i), cy = L::cy(i), c2 = cx * cx + cy * cy;
-        const long long p = fx_of<kFxTop>(get(i), emax), m = fx_of<kFxTop>(get(i + 1), emax), e = p + m, o = p - m;
+        const long long p = of(get(i)), m = of(get(i + 1)), e = p + m, o = p - m;
         axy += (long long)(cx * cy) * e;
         if (L::THERMAL) {
             ad += (long long)(cx * cx - cy * cy) * e;
@@ -517,11 +559,16 @@ __device__ __forceinline__ void fx_neq_sums(Get&& get, int emax, double& pxy, do
     pxy = fx_double<kFxTop>(axy, emax);
     if (L::THERMAL) {
         dxy = fx_double<kFxTop>(ad, emax);
-        // sums below 100 units of 2^(kFxTop + 1), the constant below 2^58
-        constexpr long long K = (long long)((5.0 - 4.0 * L::CS2) * double(1LL << 56));
-        const __int128 half = (__int128)1 << 55;
-        rx = fx_double<kFxTop>(ax + (long long)(((__int128)jx * K + half) >> 56), emax);
-        ry = fx_double<kFxTop>(ay + (long long)(((__int128)jy * K + half) >> 56), emax);
+        // the constant in units of 2^-60 (below 2^62); the product's part alone
+        // may leave 64 bits, the sum does not
+        constexpr FxCs2<LAT> C{};
+        constexpr long long K = (5LL << 60) - 4 * C.c;
+        const __int128 half = (__int128)1 << 59;
+        auto third = [&](long long a, long long j) {
+            return (long long)((unsigned long long)a + (unsigned long long)(((__int128)j * K + half) >> 60));
+        };
+        rx = fx_double<kFxTop>(third(ax, jx), emax);
+        ry = fx_double<kFxTop>(third(ay, jy), emax);
         pxx = pyy = 0.0;
     } else {
         pxx = fx_double<kFxTop>(axx, emax);
